@@ -285,8 +285,8 @@ sd_status sd_dp_psf_trace_backward(const sd_lens* const* lenses, int n_lenses,
  * (sd_dp_psf_trace_batched_workspace bytes) is device memory of the caller.
  */
 typedef struct sd_batch_config {
-  int32_t threads;        /* threads per block, multiple of 32 in 64..1024 (0 = 512) */
-  int32_t rays_per_item;  /* target rays per work item (0 = 16384) */
+  int32_t threads;        /* threads per block, multiple of 32 in 64..1024 (0 = 1024) */
+  int32_t rays_per_item;  /* target rays per work item (0 = 8192) */
   int32_t blocks_per_sm;  /* persistent blocks per SM (0 = 1) */
   int32_t reserved;
 } sd_batch_config;

@@ -2285,8 +2285,12 @@ sd_status sd_dp_psf_trace_batched(const sd_lens* const* lenses, int n_lenses,
   if (!workspace || workspace_bytes < batch_ws_bytes(n_req, total_elems)) return SD_ERR_ARG;
   sd_batch_config c{};
   if (cfg) c = *cfg;
-  if (c.threads == 0) c.threads = 512;
-  if (c.rays_per_item == 0) c.rays_per_item = 16384;
+  // one block of 1024 threads per SM: a 127 x 127 patch (129 KB) leaves room
+  // for one block, and 512 threads left half the warps idle; smaller items
+  // even out the blocks' last ones (4096 requests 4.30 -> 3.72 ms, 40 requests
+  // 0.174 -> 0.105 ms; 4096 rays an item 3.97, 16384 3.75)
+  if (c.threads == 0) c.threads = 1024;
+  if (c.rays_per_item == 0) c.rays_per_item = 8192;
   if (c.blocks_per_sm == 0) c.blocks_per_sm = 1;
   if (c.threads % 32 || c.threads < 64 || c.threads > 1024 || c.rays_per_item < 1 ||
       c.blocks_per_sm < 1 || c.blocks_per_sm > 8)
