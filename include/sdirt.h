@@ -115,6 +115,10 @@ sd_status sd_lens_paraxial(const sd_lens* lens, double lambda_nm,
  * pupil) from the changed lens.  Host call; synchronous. */
 sd_status sd_lens_set_param(sd_lens* lens, int param_id, double value);
 
+/* Changes n parameters (param_ids[i] to values[i], in order) with one upload;
+ * the lens is unchanged when one of them is refused.  Host call; synchronous. */
+sd_status sd_lens_set_params(sd_lens* lens, int n, const int* param_ids, const double* values);
+
 sd_status sd_lens_free(sd_lens* lens);
 
 /* ------------------------------------------------------------------------

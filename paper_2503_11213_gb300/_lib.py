@@ -73,7 +73,8 @@ REQUEST_DTYPE = np.dtype([("h_mm", "<f8"), ("depth_mm", "<f8"), ("lambda_nm", "<
 assert REQUEST_DTYPE.itemsize == 56
 
 # every exported symbol of include/sdirt.h
-EXPORTS = ("sd_lens_load", "sd_lens_paraxial", "sd_lens_set_param", "sd_lens_free",
+EXPORTS = ("sd_lens_load", "sd_lens_paraxial", "sd_lens_set_param",
+           "sd_lens_set_params", "sd_lens_free",
            "sd_dp_psf_trace", "sd_dp_psf_trace_backward", "sd_dp_psf_trace_mask_bytes",
            "sd_dp_psf_trace_batched",
            "sd_dp_psf_trace_batched_workspace", "sd_dp_psf_trace_batched_tune",
@@ -120,6 +121,7 @@ def lib():
     L.sd_lens_load.argtypes = [P(SdSurface), i32, dbl, P(vp)]
     L.sd_lens_paraxial.argtypes = [vp, dbl, dbl, P(SdParaxial)]
     L.sd_lens_set_param.argtypes = [vp, i32, dbl]
+    L.sd_lens_set_params.argtypes = [vp, i32, P(i32), P(dbl)]
     L.sd_lens_free.argtypes = [vp]
     L.sd_dp_psf_trace.argtypes = [P(vp), i32, P(SdSensor), vp, i32, P(SdTraceOpts), vp, vp, vp]
     L.sd_dp_psf_trace_backward.argtypes = [P(vp), i32, P(SdSensor), vp, i32, P(SdTraceOpts),

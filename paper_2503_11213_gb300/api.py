@@ -83,6 +83,15 @@ class Lens:
         L.check(L.lib().sd_lens_set_param(self.handle, int(param_id), float(value)),
                 "sd_lens_set_param")
 
+    def set_params(self, param_ids, values):
+        """set_param of several parameters with one upload."""
+        n = len(param_ids)
+        if len(values) != n:
+            raise ValueError("one value per parameter id")
+        L.check(L.lib().sd_lens_set_params(self.handle, n, (ctypes.c_int * n)(*param_ids),
+                                           (ctypes.c_double * n)(*values)),
+                "sd_lens_set_params")
+
     def free(self):
         if self._h is not None:
             L.lib().sd_lens_free(self._h)

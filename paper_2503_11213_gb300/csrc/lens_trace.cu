@@ -317,25 +317,36 @@ sd_status sd_lens_paraxial(const sd_lens* lens, double lambda_nm, double depth_m
   return SD_OK;
 }
 
-sd_status sd_lens_set_param(sd_lens* lens, int pid, double value) {
+sd_status sd_lens_set_params(sd_lens* lens, int n, const int* pids, const double* values) {
   using namespace sd;
-  if (!lens || !std::isfinite(value)) return SD_ERR_ARG;
-  DevLens& L = lens->img;
-  int s = pid / 8, j = pid % 8;
-  if (pid < 0 || s >= L.n) return SD_ERR_ARG;
-  HostExtra& X = g_extra[lens->slot];
-  if (L.type[s] == SD_SURF_STOP && j != 7) return SD_ERR_ARG;
-  if (j == 0)
-    L.c[s] = value;
-  else if (j == 1)
-    X.k[s] = value;
-  else if (j == 7) {
-    if (value < 0 || (s == L.n - 1 && value <= 0)) return SD_ERR_LENS;
-    L.t[s] = value;
-  } else
-    X.a[s][j - 2] = value;
+  if (!lens || n < 0 || (n > 0 && (!pids || !values))) return SD_ERR_ARG;
+  if (n == 0) return SD_OK;
+  DevLens L = lens->img;
+  HostExtra X = g_extra[lens->slot];
+  for (int i = 0; i < n; ++i) {
+    const double value = values[i];
+    if (!std::isfinite(value)) return SD_ERR_ARG;
+    const int pid = pids[i], s = pid / 8, j = pid % 8;
+    if (pid < 0 || s >= L.n) return SD_ERR_ARG;
+    if (L.type[s] == SD_SURF_STOP && j != 7) return SD_ERR_ARG;
+    if (j == 0)
+      L.c[s] = value;
+    else if (j == 1)
+      X.k[s] = value;
+    else if (j == 7) {
+      if (value < 0 || (s == L.n - 1 && value <= 0)) return SD_ERR_LENS;
+      L.t[s] = value;
+    } else
+      X.a[s][j - 2] = value;
+  }
   finish_image(L, X);
+  lens->img = L;
+  g_extra[lens->slot] = X;
   return upload(lens);
+}
+
+sd_status sd_lens_set_param(sd_lens* lens, int pid, double value) {
+  return sd_lens_set_params(lens, 1, &pid, &value);
 }
 
 sd_status sd_lens_free(sd_lens* lens) {
