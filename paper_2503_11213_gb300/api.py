@@ -396,9 +396,16 @@ def dp_render(aif, depth_m, bank, layout: BankLayout, out=None):
     if bank.dtype != layout.dtype or depth_m.dtype != torch.float32:
         raise ValueError("bank dtype must match the layout; depth must be float32")
     lay = layout.c()
-    L.check(L.lib().sd_dp_render(_ptr(aif), _ptr(depth_m), _ptr(bank), ctypes.byref(lay),
-                                 N, C, H, W, _DT[aif.dtype], _ptr(out), _stream()),
+    n = ctypes.c_size_t(0)
+    L.check(L.lib().sd_dp_render_workspace(ctypes.byref(lay), N, C, H, W, ctypes.byref(n)),
             "sd_dp_render")
+    try:
+        ws = torch.empty(n.value, dtype=torch.uint8, device=aif.device) if n.value else None
+    except torch.cuda.OutOfMemoryError:
+        ws = None  # no room for the re-laid bank: rendered from the bank itself
+    L.check(L.lib().sd_dp_render_ws(_ptr(aif), _ptr(depth_m), _ptr(bank), ctypes.byref(lay),
+                                    N, C, H, W, _DT[aif.dtype], _ptr(out), _ptr(ws), n.value,
+                                    _stream()), "sd_dp_render")
     return out
 
 
