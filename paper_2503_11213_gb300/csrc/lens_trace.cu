@@ -381,6 +381,7 @@ struct TraceParams {
   int map_H, map_W;
   double map_lambda_nm;
   int map_n, map_ks;
+  size_t map_slot;     // bytes of a pixel's output that map_prep_kernel filled (0: none)
   int slots[SD_MAX_LENSES];
   int n_lenses;
   SensorF sen;
@@ -401,6 +402,7 @@ struct TraceParams {
 
 // Per-request context computed by the block prologue.
 struct ReqCtx {
+  // (the nine floats are copied as a run: setup_request)
   float x_o, y_o;       // object point (x, y)
   float scale;          // pupil sample spacing r_ep / N
   float vz;             // z_ep + depth (axial length from p to the EP plane)
@@ -408,6 +410,7 @@ struct ReqCtx {
   float xc, yc;
   int slot, N, ks, total;
   int ok;
+  long long off;        // out_offset
   float eta[SD_MAX_SURFACES];    // n_before / n_after at the request wavelength
   float omeg2[SD_MAX_SURFACES];  // 1 - eta^2 (evaluated in FP64)
 };
@@ -451,42 +454,166 @@ __device__ __forceinline__ sd_psf_request request_of(const TraceParams& P, int r
   return q;
 }
 
-// Block prologue: paraxial set-up (FP64, thread 0) and pupil row tables.
-__device__ void setup_request(const TraceParams& P, const sd_psf_request& q,
-                              ReqCtx& ctx, int* prefix, int* lo) {
-  if (threadIdx.x == 0) {
-    int li = q.lens;
-    ctx.ok = (li >= 0 && li < P.n_lenses && q.n_grid >= 2 && q.n_grid <= P.max_n &&
-              q.ks >= 1 && (q.ks & 1) && q.ks <= P.max_ks && q.depth_mm > 0 &&
-              q.lambda_nm > 0);
-    if (ctx.ok) {
-      int slot = P.slots[li];
-      const DevLens& L = c_lens[slot];
-      double nlam[SD_MAX_SURFACES];
-      indices_at(L, q.lambda_nm, nlam);
-      double nb = 1.0;
-      for (int s = 0; s < L.n; ++s) {
-        double e = nb / nlam[s];
-        ctx.eta[s] = (float)e;
-        ctx.omeg2[s] = (float)(1.0 - e * e);
-        nb = nlam[s];
+// Paraxial set-up of request q (FP64) by one warp; every lane calls it.  FP64
+// runs at a few operations per clock and SM here, with the latency to match
+// (one thread doing all of it took 36 us for a 12-surface lens, 14 us for a
+// singlet), so what is independent is spread over
+// the lanes: the indices and ratios of the surfaces, the two paraxial rays
+// that locate the entrance pupil, and the divisions at the end (26 and
+// 12 us, of which each remaining division is about 1.4).
+// The operations on each value are those of ray_gen, in its order: the same
+// bits.  nl: SD_MAX_SURFACES doubles of shared memory.
+struct Pupil {
+  double z_ep, r_ep;
+};
+// The lens at one wavelength: indices (nl), ratios and the entrance pupil.
+__device__ __forceinline__ Pupil setup_lens(const DevLens& L, double lambda_nm, double* nl,
+                                            float* eta, float* omeg2) {
+  const int lane = threadIdx.x & 31;
+  const double lam = lambda_nm * 1e-3;
+  double n_s = 1.0;
+  if (lane < L.n) {
+    n_s = cauchy(L.A[lane], L.B[lane], lam);
+    nl[lane] = n_s;
+  }
+  double nb = __shfl_up_sync(0xffffffffu, n_s, 1);
+  if (lane == 0) nb = 1.0;
+  if (lane < L.n) {
+    const double e = nb / n_s;
+    eta[lane] = (float)e;
+    omeg2[lane] = (float)(1.0 - e * e);
+  }
+  __syncwarp();
+  // lane 0: the ray (1, 0) to the stop, the others (0, 1)
+  const PYU ab = parax(L, nl, lane == 0 ? 1.0 : 0.0, lane == 0 ? 0.0 : 1.0, 0, L.stop);
+  const double ay = __shfl_sync(0xffffffffu, ab.y, 0), by = __shfl_sync(0xffffffffu, ab.y, 1);
+  const double d0 = (lane == 0 ? by : L.sd_stop) / ay;
+  Pupil u;
+  u.z_ep = __shfl_sync(0xffffffffu, d0, 0);
+  u.r_ep = fabs(__shfl_sync(0xffffffffu, d0, 1));
+  return u;
+}
+
+__device__ __forceinline__ double start_plane(const DevLens& L, double z_ep) {
+  return (z_ep <= L.z_front) ? z_ep : L.z_front - 1.0;
+}
+
+__device__ __forceinline__ void setup_optics(const DevLens& L, const sd_psf_request& q,
+                                             ReqCtx& ctx, double* nl) {
+  const int lane = threadIdx.x & 31;
+  const Pupil ep = setup_lens(L, q.lambda_nm, nl, ctx.eta, ctx.omeg2);
+  const double z_ep = ep.z_ep, r_ep = ep.r_ep;
+  const double u0 = -1.0 / (z_ep + q.depth_mm);
+  const double m = parax(L, nl, 1.0 + u0 * q.depth_mm, u0, 0, L.n).y;
+  const double z_start = start_plane(L, z_ep);
+  const double num = lane == 0 ? q.h_mm : lane == 1 ? q.v_mm : lane == 2 ? r_ep : z_start + q.depth_mm;
+  const double den = lane < 2 ? m : lane == 2 ? (double)q.n_grid : z_ep + q.depth_mm;
+  const float f = (float)(num / den);
+  if (lane == 0) {
+    ctx.x_o = f;
+    ctx.vz = (float)(z_ep + q.depth_mm);
+    ctx.z_ep = (float)z_ep;
+    ctx.z_start = (float)z_start;
+    ctx.xc = (float)q.h_mm;
+    ctx.yc = (float)q.v_mm;
+  } else if (lane == 1) {
+    ctx.y_o = f;
+  } else if (lane == 2) {
+    ctx.scale = f;
+  } else if (lane == 3) {
+    ctx.s_start = f;
+  }
+}
+
+// A map's pixels share the lens, wavelength and grid; map_prep_kernel leaves
+// each one's set-up in the pixel's own output slot (which its block reads
+// before it writes the PSF there): 9 floats as in ReqCtx, eta, omeg2.
+__host__ __device__ inline int prep_floats(int n_surf) { return 9 + 2 * n_surf; }
+__device__ __forceinline__ float* prep_slot(const TraceParams& P, int r) {
+  return reinterpret_cast<float*>(reinterpret_cast<char*>(P.out) + (size_t)r * P.map_slot);
+}
+
+// Set-up of a map's pixels, one thread each: full warps on the FP64 units,
+// where a pixel's own block waits out the latency of a division and a few
+// more dependent operations per surface.  393,216 pixels of 64 x 64 grids
+// through 12 surfaces 77.4 -> 70.4 ms (of 2 x 2 grids, all set-up, 24.0 -> 6.3).
+__global__ void __launch_bounds__(128) map_prep_kernel(const TraceParams P) {
+  __shared__ double s_nl[SD_MAX_SURFACES], s_ep[2];
+  __shared__ float s_ratio[2][SD_MAX_SURFACES];
+  const DevLens& L = c_lens[P.slots[0]];
+  if (threadIdx.x < 32) {
+    const Pupil ep = setup_lens(L, P.map_lambda_nm, s_nl, s_ratio[0], s_ratio[1]);
+    if (threadIdx.x == 0) {
+      s_ep[0] = ep.z_ep;
+      s_ep[1] = ep.r_ep;
+    }
+  }
+  __syncthreads();
+  const int r = blockIdx.x * 128 + threadIdx.x;
+  if (r >= P.n_req || !(P.map_depth[r] > 0.f)) return;
+  const sd_psf_request q = request_of(P, r);
+  const double z_ep = s_ep[0], r_ep = s_ep[1];
+  const double u0 = -1.0 / (z_ep + q.depth_mm);
+  const double m = parax(L, s_nl, 1.0 + u0 * q.depth_mm, u0, 0, L.n).y;
+  const double z_start = start_plane(L, z_ep);
+  float* dst = prep_slot(P, r);
+  dst[0] = (float)(q.h_mm / m);
+  dst[1] = (float)(q.v_mm / m);
+  dst[2] = (float)(r_ep / q.n_grid);
+  dst[3] = (float)(z_ep + q.depth_mm);
+  dst[4] = (float)z_start;
+  dst[5] = (float)((z_start + q.depth_mm) / (z_ep + q.depth_mm));
+  dst[6] = (float)z_ep;
+  dst[7] = (float)q.h_mm;
+  dst[8] = (float)q.v_mm;
+  for (int i = 0; i < L.n; ++i) {
+    dst[9 + i] = s_ratio[0][i];
+    dst[9 + L.n + i] = s_ratio[1][i];
+  }
+}
+
+__device__ __forceinline__ bool valid_request(const TraceParams& P, const sd_psf_request& q) {
+  return q.lens >= 0 && q.lens < P.n_lenses && q.n_grid >= 2 && q.n_grid <= P.max_n &&
+         q.ks >= 1 && (q.ks & 1) && q.ks <= P.max_ks && q.depth_mm > 0 && q.lambda_nm > 0;
+}
+
+// Block prologue: paraxial set-up of request r (warp 0) and pupil row tables.
+// one: the request itself, where it is not the launch's r-th (hit dump).
+__device__ void setup_request(const TraceParams& P, int r, ReqCtx& ctx, int* prefix, int* lo,
+                              const sd_psf_request* one = nullptr) {
+  __shared__ double s_nl[SD_MAX_SURFACES];
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    bool ok;
+    int slot, n_grid, ks;
+    long long off;
+    if (P.map_slot) {
+      ok = P.map_depth[r] > 0.f;  // the other checks hold for every pixel
+      slot = P.slots[0];
+      n_grid = P.map_n;
+      ks = P.map_ks;
+      off = (long long)r * 2 * ks * ks;
+      if (ok) {
+        const float* src = prep_slot(P, r);
+        const int n = c_lens[slot].n;
+        for (int i = lane; i < prep_floats(n); i += 32)
+          *(i < 9 ? &ctx.x_o + i : i < 9 + n ? &ctx.eta[i - 9] : &ctx.omeg2[i - 9 - n]) = src[i];
       }
-      RayGen g = ray_gen(L, nlam, q.h_mm, q.depth_mm);
-      ctx.x_o = (float)g.x_o;
-      ctx.y_o = (float)(q.v_mm / g.m);
-      ctx.scale = (float)(g.r_ep / q.n_grid);
-      ctx.vz = (float)(g.z_ep + q.depth_mm);
-      ctx.z_ep = (float)g.z_ep;
-      ctx.z_start = (float)g.z_start;
-      ctx.s_start = (float)((g.z_start + q.depth_mm) / (g.z_ep + q.depth_mm));
-      ctx.xc = (float)q.h_mm;
-      ctx.yc = (float)q.v_mm;
-      ctx.slot = slot;
-      ctx.N = q.n_grid;
-      ctx.ks = q.ks;
     } else {
-      ctx.N = 0;
-      ctx.ks = 0;
+      const sd_psf_request q = one ? *one : request_of(P, r);
+      ok = valid_request(P, q);
+      slot = ok ? P.slots[q.lens] : 0;
+      n_grid = q.n_grid;
+      ks = q.ks;
+      off = q.out_offset;
+      if (ok) setup_optics(c_lens[slot], q, ctx, s_nl);
+    }
+    if (lane == 0) {
+      ctx.ok = ok;
+      ctx.off = off;
+      ctx.slot = slot;
+      ctx.N = ok ? n_grid : 0;
+      ctx.ks = ok ? ks : 0;
     }
   }
   __syncthreads();
@@ -1125,9 +1252,8 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
   float* patchf = reinterpret_cast<float*>(patch);
 
   const int r = blockIdx.x;
-  const sd_psf_request q = request_of(P, r);
   if (threadIdx.x < SD_N_STATS) s_stats[threadIdx.x] = 0;
-  setup_request(P, q, ctx, prefix, lo);
+  setup_request(P, r, ctx, prefix, lo);
   const int ks = ctx.ks, ks2 = ks * ks;
   for (int i = threadIdx.x; i < 2 * ks2; i += blockDim.x) patch[i] = 0u;
   const int nsurf = ctx.N ? c_lens[ctx.slot].n : 0;
@@ -1225,7 +1351,7 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
     scl = scr = total > 0 ? 1.f / (float)total : 0.f;
   }
   if (ctx.N) {
-    long long base = q.out_offset;
+    const long long base = ctx.off;
     for (int i = threadIdx.x; i < 2 * ks2; i += blockDim.x) {
       float v = (MODE == 0) ? (float)patch[i] : patchf[i];
       store_out<OutT>(P.out, base + i, v * (i < ks2 ? scl : scr));
@@ -1244,7 +1370,7 @@ __global__ void __launch_bounds__(256) trace_hits_kernel(TraceParams P, sd_psf_r
   __shared__ ReqCtx ctx;
   int* prefix = reinterpret_cast<int*>(smem);
   int* lo = prefix + (P.max_n + 1);
-  setup_request(P, q, ctx, prefix, lo);
+  setup_request(P, 0, ctx, prefix, lo, &q);
   const SensorF S = P.sen;
   const int ks = ctx.ks, p = (ks - 1) >> 1;
   const int total = ctx.N ? ctx.total : 0;
@@ -1404,6 +1530,16 @@ sd_status sd_dp_psf_map(const sd_lens* lens, const sd_dp_sensor* sensor,
   P.stats = reinterpret_cast<long long*>(stats);
   size_t smem = trace_smem_bytes(n_grid, ks);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  // the set-up in a kernel of its own, left in the output: where a pixel's
+  // PSF has room for it, and the map has more pixels than the GPU holds blocks
+  // (a launch more; below, the blocks' own set-ups run side by side)
+  const size_t pixel = (size_t)2 * ks * ks * (opts->out_dtype == SD_F32 ? 4 : 2);
+  if (pixel >= (size_t)prep_floats(lens->img.n) * 4 && (long long)H * W > 1024 &&
+      (reinterpret_cast<uintptr_t>(out) & 3) == 0) {
+    P.map_slot = pixel;
+    map_prep_kernel<<<(unsigned)(((long long)H * W + 127) / 128), 128, 0, s>>>(P);
+    if ((st = launch_status()) != SD_OK) return st;
+  }
 #define SD_LAUNCH(MODE, T)                                                          \
   do {                                                                              \
     auto kfn = trace_bin_kernel<MODE, T>;                                           \
@@ -1687,15 +1823,14 @@ __global__ void __launch_bounds__(NT, 3) trace_adj_kernel(TraceParams P, const f
   float* Gs = reinterpret_cast<float*>(smem + table_bytes(P.max_n));
   const int r = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const sd_psf_request q = request_of(P, r);
   for (int i = threadIdx.x; i < NW * SD_MAX_SURFACES * NPAR_SURF; i += NT)
     (&s_acc[0][0][0])[i] = 0.f;
   if (threadIdx.x < 2) s_swept[threadIdx.x] = 0;
-  setup_request(P, q, ctx, prefix, lo);
+  setup_request(P, r, ctx, prefix, lo);
   const int ks = ctx.ks, ks2 = ks * ks, pp = (ks - 1) >> 1;
   bool nz = false;
   for (int i = threadIdx.x; i < 2 * ks2; i += NT) {
-    const float g = G[q.out_offset + i];
+    const float g = G[ctx.off + i];
     Gs[i] = g;
     nz = nz || g != 0.f;
   }
@@ -2036,23 +2171,22 @@ __global__ void __launch_bounds__(128) prep_kernel(TraceParams P, BatchWs W, int
   int* prefix = reinterpret_cast<int*>(smem);
   int* lo = prefix + (P.max_n + 1);
   const int r = blockIdx.x;
-  const sd_psf_request q = request_of(P, r);
-  setup_request(P, q, ctx, prefix, lo);
+  setup_request(P, r, ctx, prefix, lo);
   const int ks2 = ctx.ks * ctx.ks;
-  const bool fits = ctx.N && q.out_offset >= 0 && q.out_offset + 2LL * ks2 <= total_elems;
+  const bool fits = ctx.N && ctx.off >= 0 && ctx.off + 2LL * ks2 <= total_elems;
   if (threadIdx.x == 0) {
     BatchCtx b;
     b.c = ctx;
     if (!fits) b.c.N = 0;
     b.rows_per_item = max(1, rays_per_item / max(1, ctx.N));
     b.n_items = fits ? (traced_rows(ctx) + b.rows_per_item - 1) / b.rows_per_item : 0;
-    b.off = q.out_offset;
+    b.off = ctx.off;
     W.ctx[r] = b;
     W.item_start[r] = b.n_items;  // counts; scanned by item_scan_kernel
     W.done[r] = 0u;
   }
   if (fits)
-    for (int i = threadIdx.x; i < 2 * ks2; i += blockDim.x) W.counts[q.out_offset + i] = 0u;
+    for (int i = threadIdx.x; i < 2 * ks2; i += blockDim.x) W.counts[ctx.off + i] = 0u;
   // the items OR their rays' landing bits into the request's mask words
   if (fits && P.land_mask)
     for (int i = threadIdx.x; i < (ctx.total + 31) >> 5; i += blockDim.x)
