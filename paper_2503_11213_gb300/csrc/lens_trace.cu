@@ -1111,6 +1111,14 @@ __device__ __forceinline__ bool mirrored_rays(const ReqCtx& ctx) {
   return ctx.y_o == 0.f && ctx.yc == 0.f;
 }
 
+// A round of 2 nt rays is traced as pairs (k, k + nt); the last round's `left`
+// rays as pairs (k, k + half), half a multiple of 32, so that its warps are
+// full pairs too (a 64 x 64 grid's last 156 rays: 3 warps instead of 5;
+// 512 x 768 RF50 map 70.3 -> 69.0 ms, 4096 uneven requests 3.63 -> 3.55 ms).
+__device__ __forceinline__ int round_half(int left, int nt) {
+  return left >= 2 * nt ? nt : min(nt, ((left + 1) / 2 + 31) & ~31);
+}
+
 // pupil rows whose rays are traced
 __device__ __forceinline__ int traced_rows(const ReqCtx& ctx) {
   return mirrored_rays(ctx) ? (ctx.N + 1) >> 1 : ctx.N;
@@ -1290,7 +1298,9 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
     };
     int row0 = 0, row1 = 0;
     for (int base = 0; base < traced; base += 2 * NT) {
-      const int k0 = base + threadIdx.x, k1 = k0 + NT;
+      const int half = round_half(traced - base, NT);
+      const int k0 = (int)threadIdx.x < half ? base + (int)threadIdx.x : traced;
+      const int k1 = (int)threadIdx.x < half ? k0 + half : traced;
       float2 x = make_float2(0.f, 0.f), y = x, z = x, dx = x, dy = x,
              dz = make_float2(1.f, 1.f);
       int2 st = make_int2(k0 < traced ? (int)ST_OK : (int)ST_NONE,
@@ -2400,7 +2410,9 @@ __global__ void __launch_bounds__(1024) batched_trace_kernel(TraceParams P, Batc
       // advances its own row) traced together as a packed pair
       int rw0 = 0, rw1 = 0;
       for (int base = 0; base < total; base += 2 * NT) {
-        const int k0 = base + threadIdx.x, k1 = k0 + NT;
+        const int half = round_half(total - base, NT);
+        const int k0 = (int)threadIdx.x < half ? base + (int)threadIdx.x : total;
+        const int k1 = (int)threadIdx.x < half ? k0 + half : total;
         float2 x = make_float2(0.f, 0.f), y = x, z = x, dx = x, dy = x,
                dz = make_float2(1.f, 1.f);
         int2 st = make_int2(k0 < total ? (int)ST_OK : (int)ST_NONE,
