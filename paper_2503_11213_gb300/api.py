@@ -173,7 +173,8 @@ def dp_psf_trace(lenses, sensor: DPSensor, req_dev, n_req, total, max_ks, max_n=
     if out is None:
         out = torch.empty(total, dtype=dtype, device=req_dev.device)
     if stats is None:
-        stats = torch.zeros((n_req, L.SD_N_STATS), dtype=torch.int64, device=req_dev.device)
+        # (the kernel writes every word)
+        stats = torch.empty((n_req, L.SD_N_STATS), dtype=torch.int64, device=req_dev.device)
     _need_cuda(req_dev, out, stats)
     if mask is not None and mask.numel() * 4 < land_mask_bytes(n_req, max_n):
         raise ValueError("the landing mask is too small for these requests")
@@ -230,7 +231,7 @@ def dp_psf_map(lens: Lens, sensor: DPSensor, depth_m, lambda_nm, n_grid, ks,
     if out is None:
         out = torch.empty((H, W, 2, ks, ks), dtype=dtype, device=dev)
     if stats is None:
-        stats = torch.zeros((H * W, L.SD_N_STATS), dtype=torch.int64, device=dev)
+        stats = torch.empty((H * W, L.SD_N_STATS), dtype=torch.int64, device=dev)
     _need_cuda(depth_m, out, stats)
     if depth_m.dtype != torch.float32:
         raise ValueError("depth must be float32 metres")
