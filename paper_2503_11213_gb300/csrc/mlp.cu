@@ -7,14 +7,18 @@
 // 5th-generation tensor cores:
 //   * the activations of the 128 pixels live in shared memory as the A
 //     operand (BF16, no-swizzle K-major core matrices, 128 KB);
-//   * the weights of layers 1..5 are packed on the host into 32 KB chunks of
-//     256 output rows x 64 inputs, already in the B operand layout, and one
-//     thread streams them in consumption order through a ring of three
+//   * the weights of layers 1..5 are packed on the host into 16 KB chunks of
+//     256 output rows x 32 inputs, already in the B operand layout, and two
+//     warps stream them in consumption order through a ring of five
 //     shared buffers with 1-D bulk copies (the TMA engine), completion
 //     counted in bytes on an mbarrier per buffer;
-//   * one thread issues the MMAs (M = 128, N = 256, K = 16) into a 512-column
+//   * one warp issues the MMAs (M = 128, N = 256, K = 16) into a 512-column
 //     FP32 accumulator in tensor memory and commits each buffer back to the
-//     copier;
+//     copiers.  The whole warp runs the loop and an elected lane issues, with
+//     the next chunk's barrier looked at ahead: as one lane's branch the loop
+//     took 690 cycles a chunk (clock stamps) whose products run 256, and set
+//     the kernel's time whatever the copies and epilogues did (512 x 768
+//     pixels at ks 21: 1.88 -> 1.46 ms);
 //   * eight warps (two per tensor-memory lane quarter, one per half of the
 //     columns) compute layer 0 (3 inputs, CUDA cores), and after every layer
 //     read the accumulator, add
@@ -47,7 +51,8 @@ constexpr uint32_t MCHUNK = MNC * MKC * 2;        // 16 KB
 constexpr int MKPB = MH / MKC;      // chunks per 256-row block of a layer
 constexpr uint32_t MA_BYTES = MM * MH * 2;        // 128 KB
 constexpr int MEPI = 256;           // epilogue threads: warps 0-7
-constexpr int MTHREADS = MEPI + 64;  // + warp 8 MMA issue, warp 9 copies
+constexpr int MCOPY = 2;             // copier warps
+constexpr int MTHREADS = MEPI + 32 + 32 * MCOPY;  // + warp 8 MMA issue, warps 9.. copies
 // per epilogue warp: 32 pixels x 16 outputs staged for coalesced stores
 // (rows of 18 floats: conflict-free 8-byte accesses)
 constexpr int MSROW = 18;
@@ -111,6 +116,7 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
   // written inputs 256 h .. 256 h + 255 of the next layer
   __shared__ __align__(8) uint64_t s_full[MNB], s_empty[MNB], s_acc[2], s_k0, s_epi[2], s_done;
   __shared__ uint32_t s_tmem;
+  __shared__ int s_last[MNB];  // last copy issued into each buffer
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ks = P.ks, nout = mlp_nout(ks), nblk = mlp_nblk(ks), nchunk = mlp_chunks(ks);
   const int npass = (nblk + 1) / 2;     // output passes of up to 2 x 256 columns
@@ -126,6 +132,7 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
     for (int b = 0; b < MNB; ++b) {
       tc::mbar_init(&s_full[b], 1);
       tc::mbar_init(&s_empty[b], 1);
+      s_last[b] = -1;
     }
     for (int h = 0; h < 2; ++h) {
       tc::mbar_init(&s_acc[h], 1);
@@ -140,84 +147,99 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
   tc::fence_after_sync();
   const uint32_t tmem = s_tmem;
 
-  if (warp == 9) {
-    // ---- weight copier: chunks in consumption order through the ring ------
-    if (lane == 0) {
-      int last[MNB];  // last copy issued into each buffer
-      for (int b = 0; b < MNB; ++b) last[b] = -1;
-      int c = 0;                     // copies issued
-      bool ok = true;
-      for (int ph = 0; ph < nphase && ok; ++ph) {
-        const int q = ph < 4 ? 0 : mlp_pass(ph, npass);
-        const int nb0 = ph < 4 ? 0 : 2 * q, nb1 = ph < 4 ? 2 : min(nb0 + 2, nblk);
-        for (int nb = nb0; nb < nb1 && ok; ++nb)
-          for (int kb = 0; kb < MKPB; ++kb, ++c) {
-            const int b = c % MNB;
-            if (c >= MNB && !mwait(&s_empty[b], (uint32_t)(c / MNB - 1) & 1u, P.status, P.wlim)) {
-              ok = false;
-              break;
-            }
-            // blob chunk: hidden layer ph + 1, or the output layer's block nb
-            const int chunk = (ph < 4 ? (ph * 2 + nb) * MKPB : (8 + nb) * MKPB) + kb;
+  if (warp >= 9) {
+    // ---- weight copiers: chunks in consumption order through the ring, the
+    // MCOPY warps in turn (one warp's wait and issue take longer than a chunk's
+    // products)
+    const uint32_t el = tc::elect_one();
+    int c = 0;                     // chunk
+    bool ok = true;
+    for (int ph = 0; ph < nphase && ok; ++ph) {
+      const int q = ph < 4 ? 0 : mlp_pass(ph, npass);
+      const int nb0 = ph < 4 ? 0 : 2 * q, nb1 = ph < 4 ? 2 : min(nb0 + 2, nblk);
+      for (int nb = nb0; nb < nb1 && ok; ++nb)
+        for (int kb = 0; kb < MKPB; ++kb, ++c) {
+          if (c % MCOPY != warp - 9) continue;
+          const int b = c % MNB;
+          if (c >= MNB &&
+              !__all_sync(0xffffffffu, mwait(&s_empty[b], (uint32_t)(c / MNB - 1) & 1u, P.status,
+                                             P.wlim))) {
+            ok = false;
+            break;
+          }
+          // blob chunk: hidden layer ph + 1, or the output layer's block nb
+          const int chunk = (ph < 4 ? (ph * 2 + nb) * MKPB : (8 + nb) * MKPB) + kb;
+          if (el) {
             tc::mbar_arrive_expect_tx(&s_full[b], MCHUNK);
             tc::bulk_g2s(Wbuf + (size_t)b * MCHUNK, P.blob + (size_t)chunk * MCHUNK, MCHUNK,
                          &s_full[b]);
-            last[b] = c;
           }
-      }
-      // no copy may still be landing when the CTA ends (after an error the
-      // MMA thread may not have consumed them): bounded wait for each
-      for (int b = 0; b < MNB; ++b)
-        if (last[b] >= 0) tc::mbar_wait(&s_full[b], (uint32_t)(last[b] / MNB) & 1u, MWAIT);
+          if (el) s_last[b] = c;
+        }
     }
+    // no copy may still be landing when the CTA ends (after an error the
+    // MMA warp may not have consumed them): bounded wait for each buffer's
+    // last one, by either copier
+    named_sync_m(2, 32 * MCOPY);
+    if (warp == 9)
+      for (int b = 0; b < MNB; ++b)
+        if (s_last[b] >= 0) tc::mbar_wait(&s_full[b], (uint32_t)(s_last[b] / MNB) & 1u, MWAIT);
   } else if (warp == 8) {
     // ---- MMA issue --------------------------------------------------------
-    if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16_f32(MM, MNC);
-      const uint32_t a0 = tc::smem_u32(Abuf), w0 = tc::smem_u32(Wbuf);
-      int c = 0;
-      bool ok = true;
-      // per phase: half 0 over inputs 0..255, (wait for inputs 256..511)
-      // half 0 over 256..511, half 1 over 0..255, half 1 over 256..511, so
-      // that each half's epilogue runs during the other half's MMAs
-      auto run = [&](int ph, int nb, int h, int kb0, int kb1) {
-        for (int kb = kb0; kb < kb1 && ok; ++kb, ++c) {
-          const int b = c % MNB;
-          ok = mwait(&s_full[b], (uint32_t)(c / MNB) & 1u, P.status, P.wlim);
-          if (!ok) break;
-          tc::fence_after_sync();
+    const uint32_t el = tc::elect_one();
+    const uint32_t idesc = tc::idesc_bf16_f32(MM, MNC);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint64_t ad0 = tc::smem_desc(tc::smem_u32(Abuf), 2048, 128);
+    const uint64_t bd0 = tc::smem_desc(tc::smem_u32(Wbuf), 4096, 128);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, mwait(bar, parity, P.status, P.wlim)) != 0;
+    };
+    int b = 0;               // ring buffer of the next chunk
+    uint32_t par = 0;        // and its phase
+    bool ready = false;      // already seen full
+    bool ok = true;
+    // per phase: half 0 over inputs 0..255, (wait for inputs 256..511)
+    // half 0 over 256..511, half 1 over 0..255, half 1 over 256..511, so
+    // that each half's epilogue runs during the other half's MMAs.  The next
+    // chunk's barrier is looked at before this chunk's products are issued.
+    auto run = [&](int h, int kb0, int kb1) {
+      for (int kb = kb0; kb < kb1 && ok; ++kb) {
+        if (!ready) ok = wait(&s_full[b], par);
+        if (!ok) break;
+        const int bn = b + 1 == MNB ? 0 : b + 1;
+        const uint32_t pn = par ^ (bn == 0 ? 1u : 0u);
+        const bool next = tc::mbar_test(&s_full[bn], pn);
 #pragma unroll
-          for (int s = 0; s < MKC / 16; ++s) {
-            const uint64_t ad =
-                tc::smem_desc(a0 + (uint32_t)(kb * (MKC / 8) + s * 2) * 2048u, 2048, 128);
-            const uint64_t bd =
-                tc::smem_desc(w0 + (uint32_t)b * MCHUNK + (uint32_t)s * 2 * 4096u, 4096, 128);
-            tc::mma_bf16(tmem + (uint32_t)(h * MNC), ad, bd, idesc, kb > 0 || s > 0);
-          }
-          tc::commit(&s_empty[b]);
-        }
-      };
-      for (int ph = 0; ph < nphase && ok; ++ph) {
-        const int q = ph < 4 ? 0 : mlp_pass(ph, npass);
-        const int nb0 = ph < 4 ? 0 : 2 * q;
-        const bool two = ph < 4 || nb0 + 1 < nblk;
-        ok = ok && mwait(&s_epi[0], (uint32_t)ph & 1u, P.status, P.wlim);
-        tc::fence_after_sync();
-        run(ph, nb0, 0, 0, MKPB / 2);
-        ok = ok && mwait(&s_epi[1], (uint32_t)ph & 1u, P.status, P.wlim);
-        tc::fence_after_sync();
-        run(ph, nb0, 0, MKPB / 2, MKPB);
-        tc::commit(&s_acc[0]);
-        if (two) run(ph, nb0 + 1, 1, 0, MKPB / 2);
-        tc::commit(&s_k0);
-        if (two) run(ph, nb0 + 1, 1, MKPB / 2, MKPB);
-        tc::commit(&s_acc[1]);
+        for (int s = 0; s < MKC / 16; ++s)
+          tc::mma_bf16_elect(el, tm + (uint32_t)(h * MNC),
+                             ad0 + (uint32_t)((kb * (MKC / 8) + s * 2) * (2048 / 16)),
+                             bd0 + (uint32_t)(b * (MCHUNK / 16) + s * 2 * (4096 / 16)), idesc,
+                             kb > 0 || s > 0);
+        tc::commit_elect(el, &s_empty[b]);
+        b = bn;
+        par = pn;
+        ready = __all_sync(0xffffffffu, next);
       }
-      // every MMA issued has completed before the tensor memory is freed
-      // (also after an error)
-      tc::commit(&s_done);
-      tc::mbar_wait(&s_done, 0, MWAIT);
+    };
+    for (int ph = 0; ph < nphase && ok; ++ph) {
+      const int q = ph < 4 ? 0 : mlp_pass(ph, npass);
+      const bool two = ph < 4 || 2 * q + 1 < nblk;
+      ok = ok && wait(&s_epi[0], (uint32_t)ph & 1u);
+      tc::fence_after_sync();
+      run(0, 0, MKPB / 2);
+      ok = ok && wait(&s_epi[1], (uint32_t)ph & 1u);
+      tc::fence_after_sync();
+      run(0, MKPB / 2, MKPB);
+      tc::commit_elect(el, &s_acc[0]);
+      if (two) run(1, 0, MKPB / 2);
+      tc::commit_elect(el, &s_k0);
+      if (two) run(1, MKPB / 2, MKPB);
+      tc::commit_elect(el, &s_acc[1]);
     }
+    // every MMA issued has completed before the tensor memory is freed
+    // (also after an error)
+    tc::commit_elect(el, &s_done);
+    tc::mbar_wait(&s_done, 0, MWAIT);
   } else {
     // ---- warps 0-7: layer 0, then every accumulator -------------------------
     // the two halves' sums, in the staging area (free until the first store)

@@ -73,12 +73,48 @@ __device__ __forceinline__ void mma_bf16(uint32_t taddr, uint64_t adesc, uint64_
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate));
 }
 
+// One lane of the (converged) warp.  tcgen05.mma takes its operands from
+// uniform registers: issued by a whole warp's code under this predicate, with
+// descriptors computed the same way on every lane, they stay there; issued
+// from a branch only one lane takes, every operand of every product was first
+// moved over, about 100 cycles a product where a 128 x 256 x 16 one runs 128
+// and a 128 x 64 x 16 one 32.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(e));
+  return e;
+}
+
+// mma_bf16 by the elected lane (called by the whole warp).
+__device__ __forceinline__ void mma_bf16_elect(uint32_t elected, uint32_t taddr, uint64_t adesc,
+                                               uint64_t bdesc, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected));
+}
+
 // The mbarrier at *bar completes once every previously issued tcgen05
 // operation of this thread has finished.
 __device__ __forceinline__ void commit(uint64_t* bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
           smem_u32(bar)));
+}
+
+__device__ __forceinline__ void commit_elect(uint32_t elected, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::
+          "r"(smem_u32(bar)),
+      "r"(elected));
 }
 
 // One arrival on the mbarrier (release at CTA scope).
@@ -109,6 +145,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
     if (done) return true;
   }
   return false;
+}
+
+// Whether phase `parity` of the mbarrier has completed (no waiting).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(done)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return done;
 }
 
 // Arrival that also announces tx_bytes of asynchronous copies completing on
