@@ -285,25 +285,30 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
       tc::fence_after_sync();
       if (ph < 4) {
         const float4* bias = reinterpret_cast<const float4*>(B1 + (size_t)ph * MH + half * MNC);
+        // two loads in turn: one block's latency covers the other's work
+        uint32_t r[2][32];
+        tc::tmem_ld32_issue(tbase, r[0]);
+#pragma unroll 2
         for (int c32 = 0; c32 < MNC / 32; ++c32) {
-          float bb[32], v[32];
+          uint32_t (&v)[32] = r[c32 & 1];
+          float4 bq[8];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 t = __ldg(&bias[c32 * 8 + q]);
-            bb[4 * q] = t.x;
-            bb[4 * q + 1] = t.y;
-            bb[4 * q + 2] = t.z;
-            bb[4 * q + 3] = t.w;
-          }
-          tc::tmem_ld32(tbase + (uint32_t)(c32 * 32), v);
-#pragma unroll
-          for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q] + bb[q], 0.f);
+          for (int q = 0; q < 8; ++q) bq[q] = __ldg(&bias[c32 * 8 + q]);
+          tc::tmem_wait32(v);
+          if (c32 + 1 < MNC / 32)
+            tc::tmem_ld32_issue(tbase + (uint32_t)((c32 + 1) * 32), r[(c32 + 1) & 1]);
           unsigned char* dst = Abuf + (size_t)((half * MNC) / 8 + c32 * 4) * 2048 + m * 16;
+          auto relu2 = [&](int q, float b0, float b1) {
+            return bf2(fmaxf(__uint_as_float(v[q]) + b0, 0.f),
+                       fmaxf(__uint_as_float(v[q + 1]) + b1, 0.f));
+          };
 #pragma unroll
           for (int g = 0; g < 4; ++g)
             *reinterpret_cast<uint4*>(dst + g * 2048) =
-                make_uint4(bf2(v[8 * g], v[8 * g + 1]), bf2(v[8 * g + 2], v[8 * g + 3]),
-                           bf2(v[8 * g + 4], v[8 * g + 5]), bf2(v[8 * g + 6], v[8 * g + 7]));
+                make_uint4(relu2(8 * g, bq[2 * g].x, bq[2 * g].y),
+                           relu2(8 * g + 2, bq[2 * g].z, bq[2 * g].w),
+                           relu2(8 * g + 4, bq[2 * g + 1].x, bq[2 * g + 1].y),
+                           relu2(8 * g + 6, bq[2 * g + 1].z, bq[2 * g + 1].w));
         }
         tc::fence_async_smem();
       } else {
