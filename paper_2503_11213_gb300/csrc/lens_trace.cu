@@ -704,6 +704,7 @@ __device__ __forceinline__ bool vnot(bool m) { return !m; }
 __device__ __forceinline__ M2 vnot(M2 m) { return {!m.x, !m.y}; }
 __device__ __forceinline__ bool vand(bool a, bool b) { return a && b; }
 __device__ __forceinline__ M2 vand(M2 a, M2 b) { return {a.x && b.x, a.y && b.y}; }
+__device__ __forceinline__ M2 vor(M2 a, M2 b) { return {a.x || b.x, a.y || b.y}; }
 __device__ __forceinline__ bool any_of(bool m) { return m; }
 __device__ __forceinline__ bool any_of(M2 m) { return m.x || m.y; }
 __device__ __forceinline__ float sel(bool m, float a, float b) { return m ? a : b; }
@@ -866,12 +867,22 @@ struct AdjStateV {
 };
 using AdjState = AdjStateV<float>;
 
-// A single ray returns at its first failure; a pair runs each surface to its
-// end and returns there when both rays have failed (fewer tests per ray).
-#define SD_EARLY_OUT(V, st)                          \
-  if constexpr (std::is_same<V, float>::value) {     \
-    if (dead(st)) return st;                         \
-  }
+// A single ray takes its status at once and returns at its first failure.  A
+// pair collects a surface's failure tests as predicates and looks at them
+// once at its end: only a pair with a failure takes statuses there (in the
+// tests' order), stops a failed ray at the vertex, on the axis, where no later
+// test fails, and returns when both have failed (statuses taken test by test
+// cost the ALU pipe three operations each: 3072 PSFs of 256 x 256 grids
+// 3.015 -> 2.979 ms, RF50 map 69.0 -> 68.2).
+#define SD_FAIL(V, st, flag, cond, code)             \
+  do {                                               \
+    if constexpr (std::is_same<V, float>::value) {   \
+      st = fail(st, cond, code);                     \
+      if (dead(st)) return st;                       \
+    } else {                                         \
+      flag = cond;                                   \
+    }                                                \
+  } while (0)
 
 template <bool SAVE, class V, class KS>
 __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
@@ -883,9 +894,11 @@ __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
     const SurfK<V>& S = ks_of(s);
     const int kind = S.kind;
     V t;
+    // a pair's failures at this surface: no intersection (or running
+    // backwards at a flat one), outside the aperture, total reflection
+    M f_hit{}, f_clip{}, f_tir{};
     if (kind & K_FLAT) {
-      st = fail(st, vnot(gt(dz, 0.f)), ST_BACK);
-      SD_EARLY_OUT(V, st);
+      SD_FAIL(V, st, f_hit, vnot(gt(dz, 0.f)), ST_BACK);
       t = div_nr(vneg(z), dz);
     } else {
       // conic: A t^2 - 2 B t + C = 0 (|d| = 1), root nearest the vertex in
@@ -897,13 +910,14 @@ __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
       const V disc = vfma(nA, C, vmul(B, B));
       const V den = vadd(B, sqrt_nr(disc));
       // no real root, or the root's denominator not positive
-      st = fail(st, vnot(vand(vnot(lt(disc, 0.f)), gt(den, 0.f))), ST_MISS);
-      SD_EARLY_OUT(V, st);
+      SD_FAIL(V, st, f_hit, vnot(vand(vnot(lt(disc, 0.f)), gt(den, 0.f))), ST_MISS);
       t = div_nr(C, den);
     }
     if (kind & K_ASPH) {
       // Newton on F(t) = z + t dz - sag(rho(t)^2), started at the conic root;
       // a ray stops updating t once its step is below 1e-5 mm
+      if constexpr (!std::is_same<V, float>::value)
+        st = fail(st, f_hit, (kind & K_FLAT) ? (int)ST_BACK : (int)ST_MISS);
       M act = alive(st);
       int it = 0;
       for (; it < newton_max; ++it) {
@@ -934,7 +948,11 @@ __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
         if (!any_of(act)) break;
       }
       st = fail(st, act, ST_NEWTON);  // not converged in newton_max steps
-      SD_EARLY_OUT(V, st);
+      if constexpr (std::is_same<V, float>::value) {
+        if (dead(st)) return st;
+      } else {
+        f_hit = vor(f_hit, vnot(alive(st)));
+      }
     }
     if constexpr (SAVE) sv->t[s] = t;
     x = vfma(t, dx, x);
@@ -948,8 +966,7 @@ __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
       }
     }
     const V rho2 = vfma(y, y, vmul(x, x));
-    st = fail(st, gt(rho2, S.sd2), ST_CLIP);
-    SD_EARLY_OUT(V, st);
+    SD_FAIL(V, st, f_clip, gt(rho2, S.sd2), ST_CLIP);
     if (kind & K_REFRACT) {
       V nx, ny, nz;
       if (kind & K_ASPH) {
@@ -977,15 +994,30 @@ __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
       // cos^2(t_t) = 1 - e^2 (1 - cos^2(t_i)) = (1 - e^2) + e^2 cos^2(t_i)
       const V cosi = vfma(nz, dz, vfma(ny, dy, vmul(nx, dx)));
       const V k2 = vfma(vmul(S.e2, cosi), cosi, S.om);
-      st = fail(st, lt(k2, 0.f), ST_TIR);
-      SD_EARLY_OUT(V, st);
+      SD_FAIL(V, st, f_tir, lt(k2, 0.f), ST_TIR);
       const V g = div_nr(S.om, vfma(S.e, cosi, sqrt_nr(k2)));
       dx = dot2(S.e, dx, g, nx);
       dy = dot2(S.e, dy, g, ny);
       dz = dot2(S.e, dz, g, nz);
     }
     z = vadd(z, S.negt);  // vertex-local coordinate of the next surface (or the sensor)
-    if (dead(st)) return st;
+    if constexpr (!std::is_same<V, float>::value) {
+      const M bad = vor(vor(f_hit, f_clip), f_tir);
+      if (any_of(bad)) {
+        st = fail(st, f_hit, (kind & K_FLAT) ? (int)ST_BACK : (int)ST_MISS);
+        st = fail(st, f_clip, ST_CLIP);
+        st = fail(st, f_tir, ST_TIR);
+        if (dead(st)) return st;
+        const M live = alive(st);
+        const V zero = vb<V>(0.f);
+        x = sel(live, x, zero);
+        y = sel(live, y, zero);
+        z = sel(live, z, zero);
+        dx = sel(live, dx, zero);
+        dy = sel(live, dy, zero);
+        dz = sel(live, dz, one);
+      }
+    }
   }
   st = fail(st, vnot(gt(dz, 0.f)), ST_BACK);
   if (dead(st)) return st;
