@@ -1277,10 +1277,12 @@ __device__ __forceinline__ void bin_ray(const ReqCtx& ctx, const SensorF& S, uns
 }
 
 // One block per request.  MODE 0: hard counts (u32), 1: bilinear (f32).
-// A thread traces rays k and k + blockDim.x together (packed pairs) and bins
-// each of the two sets of blockDim.x consecutive rays as one.
-template <int MODE, class OutT>
-__global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
+// A thread traces rays k and k + NT together (packed pairs) and bins each of
+// the two sets of NT consecutive rays as one.
+//   NT threads a block (1024 / NT blocks per SM, 64 registers): see
+// trace_threads.
+template <int MODE, class OutT, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) trace_bin_kernel(TraceParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ReqCtx ctx;
   __shared__ SurfK<float2> s_surf[SD_MAX_SURFACES];
@@ -1295,9 +1297,9 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
   if (threadIdx.x < SD_N_STATS) s_stats[threadIdx.x] = 0;
   setup_request(P, r, ctx, prefix, lo);
   const int ks = ctx.ks, ks2 = ks * ks;
-  for (int i = threadIdx.x; i < 2 * ks2; i += blockDim.x) patch[i] = 0u;
+  for (int i = threadIdx.x; i < 2 * ks2; i += NT) patch[i] = 0u;
   const int nsurf = ctx.N ? c_lens[ctx.slot].n : 0;
-  for (int sf = threadIdx.x; sf < nsurf; sf += blockDim.x)
+  for (int sf = threadIdx.x; sf < nsurf; sf += NT)
     s_surf[sf] = pair_consts(surf_consts(c_lens[ctx.slot].s[sf], ctx.eta[sf], ctx.omeg2[sf]));
   __syncthreads();
 
@@ -1311,11 +1313,10 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
   const bool sym = ctx.N && mirrored_rays(ctx);
   unsigned* mask = P.land_mask ? P.land_mask + (size_t)r * P.mask_words : nullptr;
   if (mask && sym) {
-    for (int i = threadIdx.x; i < (total + 31) >> 5; i += blockDim.x)
+    for (int i = threadIdx.x; i < (total + 31) >> 5; i += NT)
       if (SD_CHECK(i, P.mask_words)) mask[i] = 0u;
     __syncthreads();
   }
-  const int NT = blockDim.x;
   // one loop for each kind of request, so that the binning of mirrored rays
   // costs the other requests nothing (as run-time tests: 3.6 %)
   auto rays = [&](auto kind) {
@@ -1359,7 +1360,7 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
 
   // sums of the L and R planes for the normalisation
   float sl = 0.f, sr = 0.f;
-  for (int i = threadIdx.x; i < ks2; i += blockDim.x) {
+  for (int i = threadIdx.x; i < ks2; i += NT) {
     if (MODE == 0) {
       sl += (float)patch[i];
       sr += (float)patch[ks2 + i];
@@ -1378,7 +1379,7 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
   }
   __syncthreads();
   float SL = 0.f, SR = 0.f;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+  for (int w = 0; w < (int)(NT >> 5); ++w) {
     SL += s_red[0][w];
     SR += s_red[1][w];
   }
@@ -1394,7 +1395,7 @@ __global__ void __launch_bounds__(256, 4) trace_bin_kernel(TraceParams P) {
   }
   if (ctx.N) {
     const long long base = ctx.off;
-    for (int i = threadIdx.x; i < 2 * ks2; i += blockDim.x) {
+    for (int i = threadIdx.x; i < 2 * ks2; i += NT) {
       float v = (MODE == 0) ? (float)patch[i] : patchf[i];
       store_out<OutT>(P.out, base + i, v * (i < ks2 ? scl : scr));
     }
@@ -1441,6 +1442,17 @@ __global__ void __launch_bounds__(256) trace_hits_kernel(TraceParams P, sd_psf_r
     o[6] = side;
     o[7] = pix;
   }
+}
+
+// Threads of a request's block: with fewer requests than the GPU holds
+// 256-thread blocks, larger blocks, so that the SMs in use still hold 32 warps
+// (us, 256 threads -> more: 32 requests of a singlet at 64 x 64 27 -> 21, of a
+// 12-surface lens at 128 x 128 134 -> 87; 200 requests of that 163 -> 144, of
+// the doublet pair at 64 x 64 and ks 127 95 -> 68).  Grids below 48 x 48 have
+// too few rays for it (32 x 32: 19 -> 21).
+inline int trace_threads(int n_req, int n_sm, int max_n) {
+  if (max_n < 48 || n_req > 2 * n_sm) return 256;
+  return n_req <= n_sm ? 1024 : 512;
 }
 
 size_t trace_smem_bytes(int max_n, int max_ks) {
@@ -1518,10 +1530,15 @@ sd_status sd_dp_psf_trace(const sd_lens* const* lenses, int n_lenses,
   P.mask_words = mask_words(max_n);
   size_t smem = trace_smem_bytes(max_n, max_ks);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int threads = 256;
+  int dev = 0, n_sm = 0;
+  SD_CUDA_TRY(cudaGetDevice(&dev));
+  SD_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  const int threads = trace_threads(n_req, n_sm, max_n);
 #define SD_LAUNCH(MODE, T)                                                          \
   do {                                                                              \
-    auto kfn = trace_bin_kernel<MODE, T>;                                           \
+    auto kfn = threads == 1024 ? trace_bin_kernel<MODE, T, 1024>                    \
+               : threads == 512 ? trace_bin_kernel<MODE, T, 512>                    \
+                                : trace_bin_kernel<MODE, T, 256>;                   \
     SD_CUDA_TRY(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                      (int)smem));                                   \
     kfn<<<n_req, threads, smem, s>>>(P);                                            \
@@ -1584,7 +1601,7 @@ sd_status sd_dp_psf_map(const sd_lens* lens, const sd_dp_sensor* sensor,
   }
 #define SD_LAUNCH(MODE, T)                                                          \
   do {                                                                              \
-    auto kfn = trace_bin_kernel<MODE, T>;                                           \
+    auto kfn = trace_bin_kernel<MODE, T, 256>;                                      \
     SD_CUDA_TRY(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                      (int)smem));                                   \
     kfn<<<H * W, 256, smem, s>>>(P);                                                \

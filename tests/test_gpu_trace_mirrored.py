@@ -63,3 +63,30 @@ def test_mirrored_rays_equal_the_general_path(sdlib, mode, norm, batched):
         assert np.array_equal(x, y)
     for l in lenses:
         l.free()
+
+
+@pytest.mark.parametrize("n_req", [1, 152, 153, 304, 305])
+@pytest.mark.parametrize("v", [0.0, 0.3])
+def test_block_sizes_equal_the_batched_trace(sdlib, n_req, v):
+    """The per-request kernel's 1024, 512 and 256 threads a block (chosen by the number of requests)
+    give the batched trace's counts and masks."""
+    sd = sdlib
+    rng = np.random.default_rng(n_req)
+    reqs = np.zeros(n_req, dtype=W.REQ_DTYPE)
+    reqs["h_mm"], reqs["v_mm"] = rng.uniform(0, 1.4, n_req), v
+    reqs["depth_mm"], reqs["lambda_nm"] = rng.uniform(300, 3000, n_req), W.LAMBDA_C
+    reqs["n_grid"], reqs["ks"] = rng.integers(16, 81, n_req), rng.choice([1, 15, 65], n_req)
+    lens = sd.Lens(W.doublet_pair_f18(), 1000.0)
+    dev, total, _ = sd.make_requests(reqs)
+    masks = [sd.land_mask(n_req, 80).fill_(-1) for _ in range(2)]
+    a, sa = sd.dp_psf_trace(lens, sd.DPSensor(0.002), dev, n_req, total, max_ks=65, max_n=80,
+                            mask=masks[0])
+    bt = sd.BatchedTrace(lens, sd.DPSensor(0.002), dev, n_req, total, max_ks=65, max_n=80,
+                         mask=masks[1])
+    b, sb = bt.run()
+    torch.cuda.synchronize()
+    assert torch.equal(a, b) and torch.equal(sa, sb)
+    launched = sa[:, 0].cpu().numpy()
+    for x, y in zip(words(masks[0], reqs, launched, 80), words(masks[1], reqs, launched, 80)):
+        assert np.array_equal(x, y)
+    lens.free()
