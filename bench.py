@@ -43,9 +43,9 @@ FP32_LANES_PER_SM = 128
 # kernel, None until a capture of this build exists.  Must be re-measured
 # whenever the kernel changes.
 TRAFFIC_BYTES = {
-    # the bank and the landing mask written (63.3 MB reached DRAM within the
-    # launch), 0.7 MB read
-    "trace_bin_kernel": 64.0e6,
+    # no full-size capture of these two since they changed
+    "trace_bin_kernel": None,
+    "render_quad_kernel": None,
     # every request's gradient patch read once (also the zero patches it then
     # skips) and the landing mask of the requests it traces again: 115.5 MB
     # read + 2.0 MB written; independent of the image size
@@ -57,9 +57,6 @@ TRAFFIC_BYTES = {
     # slice bitmap 8.4 MB, work plan 0.1 MB, bank pass 47.6 MB read + 55.3 MB
     # written (the rest of the 103.8 MB gradient bank still in L2 at its end)
     "render_bwd_bank_kernel": 115.6e6,
-    # one render launch: the bank slices its tiles use and the image, 66.0 MB
-    # read, 7.9 MB of output written
-    "render_fwd_kernel": 73.9e6,
 }
 
 # ---------------------------------------------------------------------------
@@ -448,7 +445,7 @@ def run_ours(args, world, rank, local, dist):
     adj_flops = retraced_rays * fpr + swept_rays * (afr - fpr)
     phases = {  # kernel: (flops per launch, ms per launch measured on the stream)
         "trace_bin_kernel": (rays_per_step * fpr, tr_ms),
-        "render_fwd_kernel": (render_flops, rd_ms),
+        "render_quad_kernel": (render_flops, rd_ms),
         # image and bank gradients: the forward's products once each
         "render_bwd_img_kernel": (render_flops, bi_ms),
         "render_bwd_bank_kernel": (render_flops, bb_ms),
@@ -512,12 +509,12 @@ def run_ours(args, world, rank, local, dist):
         "e2e": {"value": round(e2e_value, 4), "unit": "G rays/s",
                 "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h),
                 "ms_per_step": round(e2e_ms, 4)},
-        # per step: trace; render; image gradient call (selection table,
-        # bank re-layout, two strip phases); bank gradient call (selection
-        # table, slice bitmap, slice counts, slice order, bank pass); adjoint
-        # trace and lens reduce -- 13, once in the overlapped steps and once
-        # in the sequential ones
-        "gpu_launches": 26 * args.steps,
+        # per step: trace; render (tap re-layout, render); image gradient call
+        # (selection table, bank re-layout, two strip phases); bank gradient
+        # call (selection table, slice bitmap, slice counts, slice order, bank
+        # pass); adjoint trace and lens reduce -- 14, once in the overlapped
+        # steps and once in the sequential ones
+        "gpu_launches": 28 * args.steps,
         "clocks": clocks,
         "wall_s": round(t_wall, 3),
     }
