@@ -61,7 +61,7 @@ constexpr uint32_t MWAIT = 1u << 22;
 
 __host__ __device__ inline int mlp_nout(int ks) { return 2 * ks * ks; }
 __host__ __device__ inline int mlp_nblk(int ks) { return (mlp_nout(ks) + MNC - 1) / MNC; }
-// chunks: 4 hidden layers of (512/256) x (512/64), the output layer nblk x 8
+// chunks: 4 hidden layers of (512/256) x (512/32), the output layer nblk x 16
 __host__ __device__ inline int mlp_chunks(int ks) { return 4 * 2 * MKPB + mlp_nblk(ks) * MKPB; }
 // FP32 tail: layer 0 as [512] x {w_x, w_y, w_d, b0} (one 16-byte load per
 // neuron), b1..b4 [512] each, b5 [nblk * 256]
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
   // written inputs 256 h .. 256 h + 255 of the next layer
   __shared__ __align__(8) uint64_t s_full[MNB], s_empty[MNB], s_acc[2], s_k0, s_epi[2], s_done;
   __shared__ uint32_t s_tmem;
-  __shared__ int s_last[MNB];  // last copy issued into each buffer
+  __shared__ int s_last[MCOPY][MNB];  // last copy each copier warp issued into each buffer
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ks = P.ks, nout = mlp_nout(ks), nblk = mlp_nblk(ks), nchunk = mlp_chunks(ks);
   const int npass = (nblk + 1) / 2;     // output passes of up to 2 x 256 columns
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
     for (int b = 0; b < MNB; ++b) {
       tc::mbar_init(&s_full[b], 1);
       tc::mbar_init(&s_empty[b], 1);
-      s_last[b] = -1;
+      for (int w = 0; w < MCOPY; ++w) s_last[w][b] = -1;
     }
     for (int h = 0; h < 2; ++h) {
       tc::mbar_init(&s_acc[h], 1);
@@ -174,16 +174,22 @@ __global__ void __launch_bounds__(MTHREADS, 1) mlp_kernel(const MlpParams P) {
             tc::bulk_g2s(Wbuf + (size_t)b * MCHUNK, P.blob + (size_t)chunk * MCHUNK, MCHUNK,
                          &s_full[b]);
           }
-          if (el) s_last[b] = c;
+          if (el) s_last[warp - 9][b] = c;
         }
     }
     // no copy may still be landing when the CTA ends (after an error the
     // MMA warp may not have consumed them): bounded wait for each buffer's
-    // last one, by either copier
+    // last one, by either copier.  Each copier lists its own copies, so that
+    // no word has two writers (nothing but time orders the copiers' stores
+    // before this barrier) and the wait is on the buffer's last phase
     named_sync_m(2, 32 * MCOPY);
     if (warp == 9)
-      for (int b = 0; b < MNB; ++b)
-        if (s_last[b] >= 0) tc::mbar_wait(&s_full[b], (uint32_t)(s_last[b] / MNB) & 1u, MWAIT);
+      for (int b = 0; b < MNB; ++b) {
+        int last = s_last[0][b];
+#pragma unroll
+        for (int w = 1; w < MCOPY; ++w) last = max(last, s_last[w][b]);
+        if (last >= 0) tc::mbar_wait(&s_full[b], (uint32_t)(last / MNB) & 1u, MWAIT);
+      }
   } else if (warp == 8) {
     // ---- MMA issue --------------------------------------------------------
     const uint32_t el = tc::elect_one();
