@@ -404,20 +404,31 @@ sd_status sd_dp_render(const void* aif, const float* depth_m, const void* bank,
 /*
  * sd_dp_render with a device workspace (256-byte aligned, at least
  * sd_dp_render_workspace() bytes; its contents need not be kept): the call
- * re-lays the bank's non-zero taps in it (FP32) and renders from there,
- * faster at every size.  The same sums in another order (FP32 accumulation,
- * deterministic).  A null workspace is sd_dp_render; a short or misaligned
- * one SD_ERR_ARG.
+ * re-lays the bank's non-zero taps in it (FP32) and renders from there, up to
+ * ten times faster for small images and kernels from about 21 x 21 on, and up
+ * to four times slower for small kernels on large images
+ * (sd_dp_render_advised_workspace tells which).  The same sums in another
+ * order (FP32 accumulation, deterministic).  A null workspace is
+ * sd_dp_render; a short or misaligned one SD_ERR_ARG.
  */
 sd_status sd_dp_render_ws(const void* aif, const float* depth_m, const void* bank,
                           const sd_bank_layout* layout, int N, int C, int H, int W,
                           int image_dtype, void* out, void* workspace,
                           size_t workspace_bytes, void* stream);
 
-/* Device workspace bytes of sd_dp_render_ws for these sizes: about 1.2 times
- * the bank in FP32 at ks = 65 (0 for an empty image). */
+/* Device workspace bytes of sd_dp_render_ws for these sizes (0 for an empty
+ * image): per stored slice and wavelength 2112 bytes for every 32 items, begun
+ * or full, of the (ks + 1) / 2 x ceil(ks / 4) items of 2 x 4 taps, whatever the
+ * bank's type.  That is 1.12 times the bank in FP32 at ks = 65, 3.3 times at
+ * ks = 9. */
 sd_status sd_dp_render_workspace(const sd_bank_layout* layout, int N, int C, int H, int W,
                                  size_t* bytes);
+
+/* The workspace that makes these sizes fastest: sd_dp_render_workspace's
+ * bytes where sd_dp_render_ws beats sd_dp_render, else 0 (a null workspace).
+ * Chosen by the sizes alone, from measured times. */
+sd_status sd_dp_render_advised_workspace(const sd_bank_layout* layout, int N, int C, int H,
+                                         int W, size_t* bytes);
 
 /*
  * Render from a per-pixel PSF map (supplement, "Local DP PSF convolution":

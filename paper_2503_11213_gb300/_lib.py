@@ -79,7 +79,8 @@ EXPORTS = ("sd_lens_load", "sd_lens_paraxial", "sd_lens_set_param",
            "sd_dp_psf_trace_batched",
            "sd_dp_psf_trace_batched_workspace", "sd_dp_psf_trace_batched_tune",
            "sd_dp_trace_hits", "sd_dp_psf_map",
-           "sd_dp_render", "sd_dp_render_ws", "sd_dp_render_workspace", "sd_dp_render_map", "sd_dp_render_tc", "sd_dp_render_tc_workspace", "sd_dp_render_backward",
+           "sd_dp_render", "sd_dp_render_ws", "sd_dp_render_workspace", "sd_dp_render_advised_workspace",
+           "sd_dp_render_map", "sd_dp_render_tc", "sd_dp_render_tc_workspace", "sd_dp_render_backward",
            "sd_dp_render_backward_workspace", "sd_dp_render_backward_noalloc",
            "sd_mlp_blob_bytes", "sd_mlp_pack", "sd_mlp_psf_map",
            "sd_dp_render_bank_grad_tc", "sd_dp_render_bank_grad_tc_workspace",
@@ -147,6 +148,7 @@ def lib():
     L.sd_dp_render_ws.argtypes = L.sd_dp_render.argtypes[:-1] + [vp, ctypes.c_size_t, vp]
     L.sd_dp_render_workspace.argtypes = [P(SdBankLayout), i32, i32, i32, i32,
                                          P(ctypes.c_size_t)]
+    L.sd_dp_render_advised_workspace.argtypes = L.sd_dp_render_workspace.argtypes
     L.sd_dp_render_backward.argtypes = [vp, vp, vp, vp, P(SdBankLayout), i32, i32, i32, i32,
                                         i32, vp, vp, vp, ctypes.c_size_t, vp]
     L.sd_dp_render_backward_noalloc.argtypes = [vp, vp, vp, vp, P(SdBankLayout), i32, i32, i32,

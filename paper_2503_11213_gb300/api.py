@@ -398,8 +398,10 @@ def dp_render(aif, depth_m, bank, layout: BankLayout, out=None):
         raise ValueError("bank dtype must match the layout; depth must be float32")
     lay = layout.c()
     n = ctypes.c_size_t(0)
-    L.check(L.lib().sd_dp_render_workspace(ctypes.byref(lay), N, C, H, W, ctypes.byref(n)),
-            "sd_dp_render")
+    # (0: the bank is rendered from as it is, the faster form for small kernels
+    # on large images)
+    L.check(L.lib().sd_dp_render_advised_workspace(ctypes.byref(lay), N, C, H, W,
+                                                   ctypes.byref(n)), "sd_dp_render")
     try:
         ws = torch.empty(n.value, dtype=torch.uint8, device=aif.device) if n.value else None
     except torch.cuda.OutOfMemoryError:

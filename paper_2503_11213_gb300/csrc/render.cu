@@ -29,7 +29,8 @@
 //      order of the additions cannot change the result: deterministic.
 //
 // That is the form for callers without a workspace; with one, the render goes
-// through a re-laid bank (render_quad_kernel below).
+// through a re-laid bank (render_quad_kernel below).  Each is the faster over
+// a part of the sizes: direct_is_faster.
 
 #define SD_TU 2  // translation unit id of this file's SD_CHECK sites
 #include <algorithm>
@@ -387,7 +388,8 @@ sd_status launch_fwd_cfg(RenderParams& P, cudaStream_t s) {
 // Neighbouring warps use the same slices in the same order, so most tap reads
 // hit L1.  Bound by the FMA pipe and the shared-memory and L1 reads (52
 // wavefronts per 128 FMAs).  Sums in a fixed order: deterministic.
-//   Against render_fwd_kernel (us, FP32, bank 32 x 32 but where noted):
+//   Against render_fwd_kernel (us, FP32, bank 32 x 32 but where noted; smaller
+// kernels: direct_is_faster):
 // 64 x 64 gray at ks 31 and an 8 x 4 bank 157 -> 16 (two launches); RGB at
 // ks 65: 256 x 256 1930 -> 364, 512 x 512 1630 -> 780, 8 x 512 x 512
 // 8590 -> 4990, 1024 x 1024 3077 -> 2110 (re-layout 41 of them); ks 127
@@ -678,6 +680,58 @@ sd_status launch_quad_cfg(RenderParams& P, const QuadLayout& QL, char* ws, cudaS
   return launch_status();
 }
 
+// groups of 2 x 8 pixels, each rendered by a warp or several
+inline long long quad_groups(const RenderParams& P) {
+  return (long long)((P.W + RQ_X - 1) / RQ_X) * ((P.H + RQ_R - 1) / RQ_R) * P.N * P.C;
+}
+
+// Whether render_fwd_kernel beats the render from a re-laid bank, for a caller
+// with the choice.  A warp of the re-laid form pays for a slice by whole
+// iterations of 32 items (256 taps) and a reduction of 31 shuffles, so below
+// about 17 x 17 taps its time hardly falls with ks, while the direct form's
+// does; the direct form needs images of many 128 x 32 tiles, on which few
+// slices meet (pixels a slice), and loses least to a quadrant bank, whose
+// flip classes the re-laid form selects one after the other.  The largest ks
+// at which the direct form wins was measured over banks of discs (16 x 16
+// slices, quadrant 8 x 8 x 8; FP16 the same within 3 %), by groups of 2 x 8
+// pixels (RGB but where noted; us, direct / re-laid):
+//   radial, 512 x 512 gray  ks 5 50 / 53, 7 55 / 53; 512 x 512 ks 9 114 / 130,
+//     13 144 / 133; 1024 x 1024 gray ks 15 152 / 162, 21 192 / 190;
+//     2048 x 2048 ks 3 805 / 1613, 21 1683 / 1815, 25 1919 / 1863, 65 6256 /
+//     4278;
+//   quadrant, 512 x 512 gray ks 9 60 / 80, 15 85 / 81; 1024 x 1024 ks 3 210 /
+//     661, 21 432 / 712, 33 636 / 816, 51 1016 / 1035; 2048 x 2048 ks 41
+//     2775 / 3423, 65 4940 / 4797.
+// Denser slices (1024 x 1024 with 32 x 32 of them: even at ks 15) shift it
+// down, one slice for the whole image up (1024 x 1024 gray, ks 21: 1.3 times).
+//   Both accumulate in FP32, the re-laid form in shorter chains: 4e-8 of the
+// result against FP64 at every ks, the direct form 5e-8 at ks 3, 2e-7 at ks 21
+// and 3e-7 at ks 41.
+inline bool direct_is_faster(const RenderParams& P) {
+  const long long g = quad_groups(P), slices = (long long)P.FC * P.Z;
+  int k;
+  if (P.fmode == SD_FIELD_QUADRANT)
+    k = g < 10240    ? 0
+        : g < 14336  ? 7
+        : g < 32768  ? 9
+        : g < 47104  ? 13
+        : g < 61440  ? 21
+        : g < 90112  ? 29
+        : g < 229376 ? 31
+                     : 41;
+  else
+    k = g < 14336    ? 0
+        : g < 32768  ? 5
+        : g < 53248  ? 9
+        : g < 61440  ? 13
+        : g < 131072 ? 15
+        : g < 229376 ? 17
+                     : 21;
+  if ((long long)P.H * P.W <= 256 * slices) k -= P.fmode == SD_FIELD_QUADRANT ? 4 : 2;
+  if (slices == 1) k = std::max(k, g >= 45056 ? 21 : g >= 2048 ? 7 : 0);
+  return P.ks <= k;
+}
+
 // the rows of its blocks fit the grid
 inline bool quad_fits(const RenderParams& P) { return P.H <= 65535 * RQ_R * RQ_W; }
 
@@ -709,8 +763,7 @@ sd_status launch_quad(RenderParams& P, void* workspace, cudaStream_t s) {
   // 54 / 60 / 114 / - / -, 128 x 128 168 / 135 / 149 / 163 / 197, 256 x 256
   // 571 / 431 / 364 / 438 / 450, 512 x 512 - / - / 832 / 780 / 868,
   // 1024 x 1024 - / - / 2482 / 2220 / 2137.
-  const long long groups = (long long)((P.W + RQ_X - 1) / RQ_X) * ((P.H + RQ_R - 1) / RQ_R) *
-                           P.N * P.C;
+  const long long groups = quad_groups(P);
   if (groups < 1024 && QL.maxit >= 8) return launch_quad_cfg<TI, 1, 8>(P, QL, ws, s);
   if (groups < 4096 && QL.maxit >= 4) return launch_quad_cfg<TI, 1, 4>(P, QL, ws, s);
   if (groups < 24576) return launch_quad_cfg<TI, 1, 1>(P, QL, ws, s);
@@ -722,7 +775,6 @@ constexpr size_t SMEM_CAP = 227 * 1024;
 
 template <class TI, class TB>
 sd_status launch_fwd(RenderParams& P, cudaStream_t s) {
-
   // the widest tile whose block fits in shared memory.  Up to ks = 65 the
   // kernel columns are fetched one at a time: the row extent of non-zero
   // taps is then taken per column (more empty rows skipped) and the smaller
@@ -810,6 +862,19 @@ sd_status sd_dp_render_workspace(const sd_bank_layout* layout, int N, int C, int
   const sd_status st = render_args(layout, N, C, H, W, P);
   if (st != SD_OK) return st;
   *bytes = N == 0 || H == 0 || W == 0 || !quad_fits(P) ? 0 : quad_layout(P).total;
+  return SD_OK;
+}
+
+sd_status sd_dp_render_advised_workspace(const sd_bank_layout* layout, int N, int C, int H,
+                                         int W, size_t* bytes) {
+  using namespace sd;
+  if (!bytes) return SD_ERR_ARG;
+  RenderParams P;
+  const sd_status st = render_args(layout, N, C, H, W, P);
+  if (st != SD_OK) return st;
+  *bytes = N == 0 || H == 0 || W == 0 || !quad_fits(P) || direct_is_faster(P)
+               ? 0
+               : quad_layout(P).total;
   return SD_OK;
 }
 
