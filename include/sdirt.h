@@ -408,8 +408,11 @@ sd_status sd_dp_render(const void* aif, const float* depth_m, const void* bank,
  * ten times faster for small images and kernels from about 21 x 21 on, and up
  * to four times slower for small kernels on large images
  * (sd_dp_render_advised_workspace tells which).  The same sums in another
- * order (FP32 accumulation, deterministic).  A null workspace is
- * sd_dp_render; a short or misaligned one SD_ERR_ARG.
+ * order (FP32 accumulation, deterministic).  An infinite or NaN image value
+ * reaches a pixel only through a non-zero tap; sd_dp_render also visits zero
+ * taps between, and up to seven rows above and below, the non-zero ones, where
+ * such a value gives NaN.  A null workspace is sd_dp_render; a short or misaligned
+ * one SD_ERR_ARG.
  */
 sd_status sd_dp_render_ws(const void* aif, const float* depth_m, const void* bank,
                           const sd_bank_layout* layout, int N, int C, int H, int W,

@@ -34,6 +34,7 @@
 
 #define SD_TU 2  // translation unit id of this file's SD_CHECK sites
 #include <algorithm>
+#include <type_traits>
 
 #include "render_common.cuh"
 
@@ -388,6 +389,9 @@ sd_status launch_fwd_cfg(RenderParams& P, cudaStream_t s) {
 // Neighbouring warps use the same slices in the same order, so most tap reads
 // hit L1.  Bound by the FMA pipe and the shared-memory and L1 reads (52
 // wavefronts per 128 FMAs).  Sums in a fixed order: deterministic.
+//   Blocks whose tile holds an infinite or NaN value skip the zero taps (the
+// same sums where the values are finite), so that a pixel takes such a value
+// through its non-zero taps only, whatever the items cover.
 //   Against render_fwd_kernel (us, FP32, bank 32 x 32 but where noted; smaller
 // kernels: direct_is_faster):
 // 64 x 64 gray at ks 31 and an 8 x 4 bank 157 -> 16 (two launches); RGB at
@@ -558,108 +562,124 @@ __global__ void __launch_bounds__(RQ_W * 32, 2) render_quad_kernel(
       any = any || key[g] >= 0;
     }
     if (n_class > 1 && !__syncthreads_or(any)) continue;
+    float zero = 0.f;  // NaN once an infinite or NaN value is staged
     for (int r = warp; r < P.halo_h; r += RQ_W) {
       const TI* src = img + (size_t)min(max(img_y(r - p), 0), H - 1) * W;
-      for (int i = lane; i < S; i += 32)
-        tile[r * S + i] = to_f32<TI>(__ldg(&src[min(max(img_x(i - p), 0), W - 1)]));
-    }
-    __syncthreads();
-    for (int g = 0; g < NG; ++g) {
-      int kg = key[0];
-      float tg = t[0];
-#pragma unroll
-      for (int i = 1; i < NG; ++i) {
-        kg = g == i ? key[i] : kg;
-        tg = g == i ? t[i] : tg;
+      for (int i = lane; i < S; i += 32) {
+        const float v = to_f32<TI>(__ldg(&src[min(max(img_x(i - p), 0), W - 1)]));
+        zero = fmaf(v, 0.f, zero);
+        tile[r * S + i] = v;
       }
-      const float* base = tile + row * S + g * RQ_X;
-      float tot = 0.f;  // lane l: side l & 1 of pixel l >> 1
-      int last = -1;
-      while (true) {
-        // the next slice in use: k0 unless t is 1, k0 + 1 if t is not 0
-        int cand = 0x7fffffff;
-        if (kg >= 0) {
-          if ((!two || tg < 1.f) && kg > last) cand = kg;
-          else if (two && tg > 0.f && kg + 1 > last) cand = kg + 1;
+    }
+    const bool odd = __syncthreads_or(zero != 0.f);
+    auto groups = [&](auto masked) {
+      for (int g = 0; g < NG; ++g) {
+        int kg = key[0];
+        float tg = t[0];
+#pragma unroll
+        for (int i = 1; i < NG; ++i) {
+          kg = g == i ? key[i] : kg;
+          tg = g == i ? t[i] : tg;
         }
-        const int k = (int)__reduce_min_sync(0xffffffffu, (unsigned)cand);
-        if (k == 0x7fffffff) break;
-        last = k;
-        const float w_l = kg < 0 ? 0.f : kg == k ? (two ? 1.f - tg : 1.f)
-                                     : (two && kg + 1 == k) ? tg : 0.f;
-        const size_t kl = (size_t)k * P.NL + lam;
-        const int iters = __ldg(&cnt[kl]);
-        const float4* kt = taps + (kl * QL.maxit + sub) * 128 + lane;
-        const unsigned short* kp = pos + (kl * QL.maxit + sub) * 32 + lane;
-        float2 acc[16];
+        const float* base = tile + row * S + g * RQ_X;
+        float tot = 0.f;  // lane l: side l & 1 of pixel l >> 1
+        int last = -1;
+        while (true) {
+          // the next slice in use: k0 unless t is 1, k0 + 1 if t is not 0
+          int cand = 0x7fffffff;
+          if (kg >= 0) {
+            if ((!two || tg < 1.f) && kg > last) cand = kg;
+            else if (two && tg > 0.f && kg + 1 > last) cand = kg + 1;
+          }
+          const int k = (int)__reduce_min_sync(0xffffffffu, (unsigned)cand);
+          if (k == 0x7fffffff) break;
+          last = k;
+          const float w_l = kg < 0 ? 0.f : kg == k ? (two ? 1.f - tg : 1.f)
+                                       : (two && kg + 1 == k) ? tg : 0.f;
+          const size_t kl = (size_t)k * P.NL + lam;
+          const int iters = __ldg(&cnt[kl]);
+          const float4* kt = taps + (kl * QL.maxit + sub) * 128 + lane;
+          const unsigned short* kp = pos + (kl * QL.maxit + sub) * 32 + lane;
+          float2 acc[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
-        // an iteration's item positions are loaded one ahead: the image reads
-        // wait for them (8 x 512 x 512 RGB at ks 65 5.15 -> 5.03 ms; the taps
-        // ahead as well 5.16)
-        int pk_n = sub < iters ? __ldg(kp) : 0;
-        for (int it = sub; it < iters; it += SPLIT, kt += 128 * SPLIT, kp += 32 * SPLIT) {
-          const int pk = pk_n;
-          float4 kv[4];
+          for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
+          // an iteration's item positions are loaded one ahead: the image reads
+          // wait for them (8 x 512 x 512 RGB at ks 65 5.15 -> 5.03 ms; the taps
+          // ahead as well 5.16)
+          int pk_n = sub < iters ? __ldg(kp) : 0;
+          for (int it = sub; it < iters; it += SPLIT, kt += 128 * SPLIT, kp += 32 * SPLIT) {
+            const int pk = pk_n;
+            float4 kv[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) kv[i] = __ldg(kt + 32 * i);
-          if (it + SPLIT < iters) pk_n = __ldg(kp + 32 * SPLIT);
-          const int off = (pk >> 8) * (2 * S) + (pk & 255) * 4;
-          if (!SD_CHECK(row * S + g * RQ_X + off + 2 * S + 11, P.halo_h * S)) continue;
-          const float* wp = base + off;
+            for (int i = 0; i < 4; ++i) kv[i] = __ldg(kt + 32 * i);
+            if (it + SPLIT < iters) pk_n = __ldg(kp + 32 * SPLIT);
+            const int off = (pk >> 8) * (2 * S) + (pk & 255) * 4;
+            if (!SD_CHECK(row * S + g * RQ_X + off + 2 * S + 11, P.halo_h * S)) continue;
+            const float* wp = base + off;
 #pragma unroll
-          for (int ir = 0; ir < 3; ++ir) {
-            float w[12];
+            for (int ir = 0; ir < 3; ++ir) {
+              float w[12];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-              const float4 q = *reinterpret_cast<const float4*>(wp + ir * S + 4 * i);
-              w[4 * i] = q.x;
-              w[4 * i + 1] = q.y;
-              w[4 * i + 2] = q.z;
-              w[4 * i + 3] = q.w;
-            }
+              for (int i = 0; i < 3; ++i) {
+                const float4 q = *reinterpret_cast<const float4*>(wp + ir * S + 4 * i);
+                w[4 * i] = q.x;
+                w[4 * i + 1] = q.y;
+                w[4 * i + 2] = q.z;
+                w[4 * i + 3] = q.w;
+              }
 #pragma unroll
-            for (int pr = 0; pr < 2; ++pr) {
-              const int tr = ir - pr;  // tap row of pixel row pr
-              if (tr < 0 || tr > 1) continue;
+              for (int pr = 0; pr < 2; ++pr) {
+                const int tr = ir - pr;  // tap row of pixel row pr
+                if (tr < 0 || tr > 1) continue;
 #pragma unroll
-              for (int tp = 0; tp < 4; ++tp) {
-                const float4 kq = kv[2 * tr + (tp >> 1)];
-                const float2 k2 = (tp & 1) ? make_float2(kq.z, kq.w) : make_float2(kq.x, kq.y);
+                for (int tp = 0; tp < 4; ++tp) {
+                  const float4 kq = kv[2 * tr + (tp >> 1)];
+                  const float2 k2 = (tp & 1) ? make_float2(kq.z, kq.w) : make_float2(kq.x, kq.y);
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                  acc[pr * 8 + j] =
-                      __ffma2_rn(make_float2(w[j + tp], w[j + tp]), k2, acc[pr * 8 + j]);
+                  for (int j = 0; j < 8; ++j) {
+                    const float2 f =
+                        __ffma2_rn(make_float2(w[j + tp], w[j + tp]), k2, acc[pr * 8 + j]);
+                    if (!decltype(masked)::value) {
+                      acc[pr * 8 + j] = f;
+                    } else {
+                      if (k2.x != 0.f) acc[pr * 8 + j].x = f.x;
+                      if (k2.y != 0.f) acc[pr * 8 + j].y = f.y;
+                    }
+                  }
+                }
               }
             }
           }
-        }
-        float v[32];
+          float v[32];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          v[2 * j] = acc[j].x;
-          v[2 * j + 1] = acc[j].y;
+          for (int j = 0; j < 16; ++j) {
+            v[2 * j] = acc[j].x;
+            v[2 * j + 1] = acc[j].y;
+          }
+          const float sum = warp_sum32(v);
+          const float w = __shfl_sync(0xffffffffu, w_l, lane >> 1);
+          // a pixel that does not use the slice takes nothing of it (not even
+          // 0 * inf)
+          if (w != 0.f) tot = fmaf(w, sum, tot);
         }
-        const float sum = warp_sum32(v);
-        const float w = __shfl_sync(0xffffffffu, w_l, lane >> 1);
-        // a pixel that does not use the slice takes nothing of it (not even
-        // 0 * inf)
-        if (w != 0.f) tot = fmaf(w, sum, tot);
+        if (SPLIT > 1) {  // the warps' parts added in order by the first
+          s_part[warp][lane] = tot;
+          __syncthreads();
+          if (sub == 0)
+            for (int w = 1; w < SPLIT; ++w) tot += s_part[warp + w][lane];
+        }
+        const int j = lane >> 1, side = (lane & 1) ^ (mx ? 1 : 0);
+        const int yy = img_y(row + (j >> 3)), xx = img_x(g * RQ_X + (j & 7));
+        const bool mine = __shfl_sync(0xffffffffu, kg, j) >= 0;
+        if (sub == 0 && mine && yy < H && xx < W) {
+          TI* out = reinterpret_cast<TI*>(P.out) + ((size_t)n * 2 + side) * P.C * H * W;
+          out[((size_t)c * H + yy) * W + xx] = from_f32<TI>(tot);
+        }
       }
-      if (SPLIT > 1) {  // the warps' parts added in order by the first
-        s_part[warp][lane] = tot;
-        __syncthreads();
-        if (sub == 0)
-          for (int w = 1; w < SPLIT; ++w) tot += s_part[warp + w][lane];
-      }
-      const int j = lane >> 1, side = (lane & 1) ^ (mx ? 1 : 0);
-      const int yy = img_y(row + (j >> 3)), xx = img_x(g * RQ_X + (j & 7));
-      const bool mine = __shfl_sync(0xffffffffu, kg, j) >= 0;
-      if (sub == 0 && mine && yy < H && xx < W) {
-        TI* out = reinterpret_cast<TI*>(P.out) + ((size_t)n * 2 + side) * P.C * H * W;
-        out[((size_t)c * H + yy) * W + xx] = from_f32<TI>(tot);
-      }
-    }
+    };
+    // items, and the idle lanes of a last iteration, reach past the kernel with
+    // zero taps: over an infinite value those would add NaN
+    if (odd) groups(std::true_type{}); else groups(std::false_type{});
     if (n_class > 1) __syncthreads();  // the next class stages the tile again
   }
 }
