@@ -508,9 +508,9 @@ __global__ void __launch_bounds__(IG_NW * 32, 3) render_bwd_img_kernel(
 // Work plan of a bank-gradient launch (built on the device by
 // slice_count_kernel and slice_order_kernel, in the caller's workspace).
 struct BankPlan {
-  const int* order;  // item of each block rank: key * 2 + chunk; -1 past the last
+  const int* order;  // item of each block rank: key * 2 + chunk; -1: none
   const int* slot;   // split slot of a key, -1 for a slice that is one item
-  const int* cnt;    // tiles that use a key
+  const int* cnt;    // tiles that use a key (read by a quadrant bank's fold)
   int* tick;         // per (split slot, wavelength): chunks finished
   float* pbuf;       // per (split slot, chunk, wavelength): a 2 ks^2 slab
   int nkeys;
@@ -591,7 +591,8 @@ __global__ void __launch_bounds__(256) slice_count_kernel(const unsigned* __rest
 // threads; everything it decides follows from the counts (deterministic).
 __global__ void __launch_bounds__(1024) slice_order_kernel(const int* __restrict__ cnt,
                                                            int nkeys, int NL, int resident,
-                                                           int smax, int* __restrict__ slot,
+                                                           int smax, bool used_only,
+                                                           int* __restrict__ slot,
                                                            int* __restrict__ split_key,
                                                            int* __restrict__ order) {
   constexpr int NB = 64;
@@ -687,7 +688,9 @@ __global__ void __launch_bounds__(1024) slice_order_kernel(const int* __restrict
     __syncthreads();
     if (valid) {
       const int pos = s_base[b] + s_wc[warp][b] + rank;
-      if (pos < nitems) order[pos] = item_key(id) * 2 + (id < nkeys ? 0 : 1);
+      const int key = item_key(id);
+      if (pos < nitems)
+        order[pos] = used_only && cnt[key] == 0 ? -1 : key * 2 + (id < nkeys ? 0 : 1);
     }
     __syncthreads();
     if (tid < NB) s_base[tid] += s_tot[tid];
@@ -741,9 +744,8 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 3 : (NT <= 320 ? 2 : 1)) rende
   __shared__ int s_nseg, s_wcnt[NSEG / 32];
 
   const int lam = (int)(blockIdx.x % P.NL), item = plan.order[blockIdx.x / P.NL];
-  if (item < 0 || (item >> 1) >= plan.nkeys) return;  // past the last item
+  if (item < 0 || (item >> 1) >= plan.nkeys) return;  // no item
   const int key = item >> 1, chunk = item & 1, sl = plan.slot[key], nch = sl >= 0 ? 2 : 1;
-  if (P.fmode == SD_FIELD_QUADRANT && plan.cnt[key] == 0) return;  // its slab is not folded
   const int tid = threadIdx.x;
   const bool two = P.Z > 1;
   const int nstrip = ks * (KU / SEG);
@@ -973,7 +975,8 @@ inline sd_status launch_plan(const RenderParams& P, const unsigned* bm, int word
   slice_count_kernel<<<g, 256, 0, s>>>(bm, words, ntiles, nk, cnt);
   sd_status st = launch_status();
   if (st != SD_OK) return st;
-  slice_order_kernel<<<1, 1024, 0, s>>>(cnt, nk, P.NL, resident, L.smax, slot, split, order);
+  slice_order_kernel<<<1, 1024, 0, s>>>(cnt, nk, P.NL, resident, L.smax,
+                                        P.fmode == SD_FIELD_QUADRANT, slot, split, order);
   st = launch_status();
   if (st != SD_OK) return st;
   plan->order = order;
@@ -1172,9 +1175,8 @@ __global__ void __launch_bounds__(BG_NT, 2) bank_grad_tc_kernel(
   // block (rank * NL + lam): item order[rank] (a slice or one tile chunk of
   // a split slice; the items with the most tiles first)
   const int lam = (int)(blockIdx.x % P.NL), item = plan.order[blockIdx.x / P.NL];
-  if (item < 0 || (item >> 1) >= plan.nkeys) return;  // past the last item
+  if (item < 0 || (item >> 1) >= plan.nkeys) return;  // no item
   const int key = item >> 1, chunk = item & 1, sl = plan.slot[key], nch = sl >= 0 ? 2 : 1;
-  if (P.fmode == SD_FIELD_QUADRANT && plan.cnt[key] == 0) return;  // its slab is not folded
   const bool two = P.Z > 1;
   const int kw = key >> 5;
   const unsigned kbit = 1u << (key & 31);

@@ -58,7 +58,7 @@ def test_only_non_zero_taps_take_non_finite_values(sdlib, H, W, C, ks, quadrant,
     depth = torch.ones((1, H, W), device="cuda")
     if quadrant:  # the flip classes exchange sides and mirror: render the indicators to count
         clean = torch.where(bad.any(0), torch.zeros_like(img), img)
-        ones = torch.tensor((K != 0), dtype=bank)
+        ones = (K != 0).to(bank)
         cnt = [render_ws(sd, m.to(image).cuda(), depth, ones.cuda(), lay).cpu() > 0.5 for m in bad]
         want = render_ws(sd, clean.cuda(), depth, K.cuda(), lay).cpu()
     else:
