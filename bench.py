@@ -107,10 +107,19 @@ def flops_per_ray(table):
     return f
 
 
-def in_pupil_rays(n):
-    ix = np.arange(n)
-    a = 2 * ix + 1 - n
-    return int(((a[:, None] ** 2 + a[None, :] ** 2) <= n * n).sum())
+def in_pupil_rays(n, rows=None):
+    """In-pupil samples of an n x n grid (of its first `rows` rows)."""
+    a = 2 * np.arange(n) + 1 - n
+    return int(((a[:rows, None] ** 2 + a[None, :] ** 2) <= n * n).sum())
+
+
+def traced_rays(reqs):
+    """Rays of the requests that the forward trace traces: on the sensor's x
+    axis (v = 0) those of the pupil rows up to the middle one, whose mirror
+    images stand for the rest; elsewhere all."""
+    rays = {(n, on): in_pupil_rays(n, (n + 1) // 2 if on else None)
+            for n in set(reqs["n_grid"].tolist()) for on in (False, True)}
+    return sum(rays[n, v == 0] for n, v in zip(reqs["n_grid"].tolist(), reqs["v_mm"].tolist()))
 
 
 def load_peaks():
@@ -440,11 +449,13 @@ def run_ours(args, world, rank, local, dist):
     # algorithmic work of each phase (FMA = 2 flops)
     render_flops = H * Wd * 3 * 2 * 2 * cfg["ks"] ** 2 * 2  # px, ch, L/R, 2 slices, FMA
     afr = adjoint_flops_per_ray(cfg["lens"])
-    # the adjoint: every launched ray is traced again (the forward's work),
-    # the reverse sweep counts only for the rays that carry a contribution
+    # the forward: the rays it traces; the adjoint: those it traces again (the
+    # forward's work), the reverse sweep only for the ones that carry a
+    # contribution
+    traced = traced_rays(reqs)
     adj_flops = retraced_rays * fpr + swept_rays * (afr - fpr)
     phases = {  # kernel: (flops per launch, ms per launch measured on the stream)
-        "trace_bin_kernel": (rays_per_step * fpr, tr_ms),
+        "trace_bin_kernel": (traced * fpr, tr_ms),
         "render_quad_kernel": (render_flops, rd_ms),
         # image and bank gradients: the forward's products once each
         "render_bwd_img_kernel": (render_flops, bi_ms),
@@ -497,6 +508,7 @@ def run_ours(args, world, rank, local, dist):
                      "fp32_probe": fp32,
                      "derived_peak_at_max_clock": round(derived_tflops, 2),
                      "flops_per_ray": fpr, "adjoint_flops_per_ray": afr,
+                     "traced_rays": traced,
                      "adjoint_live_request_rays": live_rays,
                      "adjoint_retraced_rays": retraced_rays,
                      "adjoint_swept_rays": swept_rays, "adjoint_swept_slots": swept_slots,
