@@ -654,8 +654,9 @@ __device__ void setup_request(const TraceParams& P, int r, ReqCtx& ctx, int* pre
 // to the compiler), and the float2 forms are the packed two-lane
 // instructions of sm_100 and later, whose components round exactly like the
 // scalar ones.  So a ray traced alone and the same ray traced as one of a
-// pair give the same bits, and the forward (pairs), the adjoint's recompute,
-// the batched trace and the map trace (single rays) take the same decisions.
+// pair give the same bits, and the forward, batched and map traces and the
+// adjoint's recompute (pairs) and the hit dump (single rays) take the same
+// decisions.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
@@ -1027,8 +1028,7 @@ __device__ __forceinline__ typename VStat<V>::S trace_ray_v(
   return st;
 }
 
-// One ray, the surface constants derived on the fly (the adjoint, the
-// batched trace, the map trace, the hit dump).
+// One ray, the surface constants derived on the fly (the hit dump).
 template <bool SAVE>
 __device__ __forceinline__ int trace_ray_t(int slot, const float* __restrict__ eta,
                                            const float* __restrict__ omeg2, int newton_max,
@@ -1448,8 +1448,11 @@ __global__ void __launch_bounds__(256) trace_hits_kernel(TraceParams P, sd_psf_r
 // 256-thread blocks, larger blocks, so that the SMs in use still hold 32 warps
 // (us, 256 threads -> more: 32 requests of a singlet at 64 x 64 27 -> 21, of a
 // 12-surface lens at 128 x 128 134 -> 87; 200 requests of that 163 -> 144, of
-// the doublet pair at 64 x 64 and ks 127 95 -> 68).  Grids below 48 x 48 have
-// too few rays for it (32 x 32: 19 -> 21).
+// the doublet pair at 64 x 64 and ks 127 95 -> 68).  The line is drawn at max_n,
+// which is all the host knows of the grids: for one of 8 to 24 samples a side it
+// does not matter much (32 requests of a singlet at 16 x 16, kernel: 13.5 with
+// 256 threads, 14.6 with 1024), and from 40 on the larger blocks win (40 x 40:
+// 16.8 and 15.4; off the axis 18.0 and 15.4).
 inline int trace_threads(int n_req, int n_sm, int max_n) {
   if (max_n < 48 || n_req > 2 * n_sm) return 256;
   return n_req <= n_sm ? 1024 : 512;

@@ -396,7 +396,7 @@ sd_status launch_fwd_cfg(RenderParams& P, cudaStream_t s) {
 // kernels: direct_is_faster):
 // 64 x 64 gray at ks 31 and an 8 x 4 bank 157 -> 16 (two launches); RGB at
 // ks 65: 256 x 256 1930 -> 364, 512 x 512 1630 -> 780, 8 x 512 x 512
-// 8590 -> 4990, 1024 x 1024 3077 -> 2110 (re-layout 41 of them); ks 127
+// 8590 -> 4990, 1024 x 1024 3077 -> 2040 (re-layout 41 of them); ks 127
 // 256 x 256 2266 -> 700.
 // ---------------------------------------------------------------------------
 constexpr int RQ_W = 8;             // warps per block

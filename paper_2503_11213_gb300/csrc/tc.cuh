@@ -73,12 +73,12 @@ __device__ __forceinline__ void mma_bf16(uint32_t taddr, uint64_t adesc, uint64_
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate));
 }
 
-// One lane of the (converged) warp.  tcgen05.mma takes its operands from
-// uniform registers: issued by a whole warp's code under this predicate, with
-// descriptors computed the same way on every lane, they stay there; issued
-// from a branch only one lane takes, every operand of every product was first
-// moved over, about 100 cycles a product where a 128 x 256 x 16 one runs 128
-// and a 128 x 64 x 16 one 32.
+// One lane of the (converged) warp.  The network's product loop, run by the
+// whole warp with the issue under this predicate, keeps ahead of its products;
+// as a branch of one lane it took 690 cycles (clock stamps) a chunk of two
+// 128 x 256 x 16 products, which run 256.  The tensor-core render and bank
+// gradient gain nothing from it (6.20 -> 6.35, 8.14 -> 8.26 ms) and issue from
+// one lane.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t e;
   asm volatile(
