@@ -389,7 +389,10 @@ class BankLayout:
 
 def dp_render(aif, depth_m, bank, layout: BankLayout, out=None):
     """aif (N,C,H,W) f32/bf16/f16, depth (N,H,W) f32 metres, bank in
-    layout.dtype -> DP image (N,2C,H,W) in aif's dtype."""
+    layout.dtype -> DP image (N,2C,H,W) in aif's dtype.  Unless the kernels are
+    small and the image large, the bank is re-laid in a workspace allocated for
+    the call (sd_dp_render_workspace: 1.1 times an FP32 bank at ks 65, 2.2 times
+    a 16-bit one); without room for it the bank is rendered from as it is."""
     N, C, H, W = aif.shape
     if out is None:
         out = torch.empty((N, 2 * C, H, W), dtype=aif.dtype, device=aif.device)

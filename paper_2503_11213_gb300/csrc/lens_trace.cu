@@ -2357,6 +2357,9 @@ __device__ void batch_flush(const TraceParams& P, const BatchWs& W, int r, int i
   __syncthreads();
 }
 
+// Both ray loops (mirrored requests and the rest) in one kernel of 64 registers
+// spill 48 B a thread; at 1024 threads it still gains off the axis, where no ray
+// is mirrored (4096 requests of 32 to 256 samples a side 4.21 -> 3.52 ms).
 template <class OutT>
 __global__ void __launch_bounds__(1024) batched_trace_kernel(TraceParams P, BatchWs W, int n_req) {
   extern __shared__ __align__(16) unsigned char smem[];
